@@ -27,7 +27,8 @@
 void blast_last_error(const char *file, int line, const char *msg);
 
 // Lets `func` launch with as much dynamic shared memory as the device allows a
-// block beside the kernel's static shared memory.  Every caller writes the same
+// block beside the kernel's static shared memory.  Called when a plan is made, not
+// per launch (it costs more host time than a launch).  Every caller writes the same
 // value, so plans served from several host threads cannot race on the
 // attribute (a per-launch size written by one thread could fall under the size
 // another thread launches with).
@@ -73,6 +74,7 @@ struct blast_plan {
     int r_form = 0;  // 0: R in [R_min, R_max]; 1: symmetrised form on (0, 1]
     double chi_min = 0, chi_max = 0, R_min = 0, R_max = 0, k_min = 0, k_max = 0;
     int max_clust = 0, max_lens = 0, max_tr = 0, device = 0;
+    int sms = 0, smem_optin = 0;    // the device's SMs and largest shared memory of a block
 
     // host grids
     std::vector<double> chi, wchi, R, wR, tcheb, kcheb;
@@ -95,6 +97,9 @@ struct blast_plan {
     float *scT = nullptr;           // [3 L Q / 32] 2^(eG - 16) per 32-column tile
     int Kmma = 0;                   // N rounded up to a multiple of 16 (the MMA's K)
     int Kst = 0;                    // stored K of the slice table: max(64, Kmma), zero padded
+    uint16_t *colexp = nullptr;     // biased exponent of the largest entry of every basis column [3 L Q]
+    int *d_slab = nullptr;          // largest of those per (type, ell)
+    bool fx_ok = false;             // the digits of the FP64 tensor-core contraction hold this basis
     bool have64 = false, have32 = false, havebf = false;
     int *d_err = nullptr;           // host-mapped error word written by bounded device waits
     int test_trip = -1;             // test hook of the tensor-core contraction (blast_test_trip_wait)
@@ -161,6 +166,12 @@ int launch_fit(blast_plan *p, ReqDev *dreq, int nreq, cudaStream_t s);
 int launch_weights(blast_plan *p, ReqDev *dreq, int nreq, int want32, cudaStream_t s, int want_v64 = 1);
 int launch_contract(blast_plan *p, ReqDev *dreq, int nreq, int prec, const int *d_esel, int n_esel,
                     void *ypart, cudaStream_t s);
+// FP64 contraction on the tensor cores (contract_fx.cu): column exponents of the
+// basis (sets p->fx_ok), and the contraction with the CUDA-core path's partials.
+int fx_prepare(blast_plan *p, cudaStream_t s);
+int launch_contract_fx(blast_plan *p, const ReqDev *dreq, int n, const int *d_esel, int n_esel, double *Y,
+                       cudaStream_t s);
+int fx_kernels(int device);
 int launch_reduce(blast_plan *p, ReqDev *dreq, int nreq, int prec, const int *d_esel, int n_esel,
                   const void *ypart, cudaStream_t s);
 int launch_contract_tc(blast_plan *p, ReqDev *dreq, int nreq, const int *d_esel, int n_esel,
@@ -201,4 +212,8 @@ int request_check(const blast_plan *p, const blast_request *r);  // the checks o
 int request_n_sel(const blast_plan *p, const blast_request *r);  // ells selected by the mask
 double host_now();
 int noalloc_prepare(int dev);     // allocation-free path: scratch address and kernel code, per device
-int preload_fp64_kernels();       // load the FP64 evaluation kernels' code (lazy module loading)
+// Set-up of the kernels on a device, by blast_plan_create: code loaded (loading is
+// lazy), shared-memory limits raised, so that a launch makes no such call.
+int preload_fp64_kernels(int device);
+int tc_kernels(int device);
+int limber_kernels(int device);

@@ -49,6 +49,7 @@
 #include <cstring>
 
 #include "blast_internal.h"
+#include "tc_ptx.h"
 
 namespace {
 
@@ -66,8 +67,6 @@ constexpr uint32_t kBSliceBytes = kQT * 128;  // 32 rows x 64 bf16
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kCtrlBytes = 256;          // mbarriers, TMEM address, abort flag
 constexpr uint32_t kEselBytes = 4 * BLAST_MAX_ELL;  // selected ells
-constexpr long long kWaitLimit = 4000000000LL;  // clock cycles (about 2 s)
-constexpr uint32_t kSuspendNs = 1000000;        // longest suspension of one phase test
 
 // Compile-time shape of one kernel instance: KC 64-wide K chunks per stage
 // (1: order <= 64, 2: order <= 96).
@@ -85,85 +84,6 @@ template <int KC> struct TcCfg {
     static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kA4Bytes + kCtrlBytes + kEselBytes +
                                     kYbufFloats * 4;
 };
-
-// ---------------------------------------------------------------- PTX helpers
-__device__ __forceinline__ uint32_t smem_u32(const void *p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-// One test of a phase; a thread that finds it incomplete is suspended until the
-// phase completes or about kSuspendNs nanoseconds pass, so waiting warps do not
-// take issue slots from working ones.
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity), "r"(kSuspendNs)
-        : "memory");
-    return ok != 0;
-}
-
-// Barrier among n threads (whole warps) of the CTA on hardware barrier id (1..15).
-__device__ __forceinline__ void named_bar_sync(int id, int n)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
-}
-
-// Bounded wait on a phase: false if it did not complete within kWaitLimit
-// cycles.  With sleep_ns > 0 the thread sleeps between tests, doubling up to
-// 1 us: for the TMA and MMA warps, which wait most of the time and need not
-// answer within a few cycles.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, unsigned sleep_ns = 0,
-                                          long long limit = kWaitLimit)
-{
-    if (mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity)) {
-        if (clock64() - t0 > limit) return false;
-        if (sleep_ns) {
-            __nanosleep(sleep_ns);
-            sleep_ns = min(2u * sleep_ns, 1024u);
-        }
-    }
-    return true;
-}
-
-__device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y, int z)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z)
-        : "memory");
-}
-
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-        ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y)
-        : "memory");
-}
 
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of
 // 128 bytes, 8-row groups 1024 bytes apart.
@@ -201,50 +121,6 @@ __device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint64_t ad, uint64_t b
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
         ::"r"(d_tmem), "l"(ad), "l"(bd), "r"(kIdesc), "r"(acc));
-}
-
-// True in exactly one lane of the (converged) warp.
-__device__ __forceinline__ bool elect_one()
-{
-    uint32_t p;
-    asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}\n" : "=r"(p));
-    return p != 0;
-}
-
-// Eight consecutive 32-bit columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
-{
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-                 : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(taddr));
-}
-
-__device__ __forceinline__ void tmem_wait_ld4(uint32_t (&r)[4])
-{
-    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]) : : "memory");
-}
-
-// Register fence for values a tcgen05.wait::ld has already covered: ties
-// them to a point after that wait.
-__device__ __forceinline__ void reg_fence4(uint32_t (&r)[4])
-{
-    asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]) : : "memory");
-}
-
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-__device__ __forceinline__ void umma_commit(uint64_t *bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                     smem_u32(bar))
-                 : "memory");
 }
 
 // Knuth's two-sum: s + e == a + b exactly, s = fl(a + b).
@@ -322,22 +198,6 @@ __device__ __forceinline__ void two_sum2(f32x2 a, f32x2 b, f32x2 &s, f32x2 &e)
     e = add2(sub2(a, sub2(ss, bb)), sub2(b, bb));
     s = ss;
 }
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// One-dimensional bulk copy global -> shared (both 16-byte aligned, size a
-// multiple of 16) completing on an mbarrier of this CTA.
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
-// Order this thread's earlier generic-proxy accesses of shared memory before
-// later async-proxy (bulk copy) writes to it.
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // ---------------------------------------------------------------- slicing
 // x (|x| < 1) -> S slices: integers in [-256, 256] times 2^(-8p) f for slice
@@ -1107,15 +967,13 @@ int launch_contract_inst(blast_plan *p, const CUtensorMap &mapB, const CUtensorM
                          cudaStream_t s)
 {
     using C = TcCfg<KC>;
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+    const int sms = p->sms;
     const int units = args.nbt * args.ngr * args.nqt;
     // persistent CTAs: the autotuned count when set, else every SM
     int grid = p->tune.grid > 0 ? p->tune.grid : sms / args.nbt * args.nbt;
     grid = grid / args.nbt * args.nbt;
     if (grid > units) grid = units;
     if (grid < args.nbt) grid = args.nbt;
-    BL_CUDA(allow_opt_in_smem(k_contract_tc<KC>, p->device));
     k_contract_tc<KC><<<grid, kThreads, C::kSmem, s>>>(mapB, mapA4, args);
     BL_CUDA(cudaGetLastError());
     return BLAST_OK;
@@ -1129,6 +987,15 @@ int launch_contract_inst(blast_plan *p, const CUtensorMap &mapB, const CUtensorM
 bool tc_supported(const blast_plan *p)
 {
     return p->Kmma <= 96 && p->Rn % kQT == 0 && p->max_clust <= 2 * kNB && p->max_lens <= 2 * kNB;
+}
+
+int tc_kernels(int device)
+{
+    BL_CUDA(allow_opt_in_smem(k_contract_tc<1>, device));
+    BL_CUDA(allow_opt_in_smem(k_contract_tc<2>, device));
+    BL_CUDA(allow_opt_in_smem(k_reduce_tc<kNB>, device));
+    BL_CUDA(allow_opt_in_smem(k_reduce_tc<2 * kNB>, device));
+    return BLAST_OK;
 }
 
 size_t tc_ws_total(const blast_plan *p, int n)
@@ -1234,12 +1101,10 @@ int launch_reduce_tc(blast_plan *p, ReqDev *dreq, int n, const int *d_esel, int 
     const size_t smem = (size_t)W * NS * stage;
     dim3 grid((n + 31) / 32, n_esel, npass * ngr);  // cosmology tiles of 32 that hold a request
     if (MT > kNB) {
-        BL_CUDA(allow_opt_in_smem(k_reduce_tc<2 * kNB>, p->device));
         k_reduce_tc<2 * kNB><<<grid, 32 * W, smem, s>>>(dreq, (const float *)ypart, U, n, p->X, p->L, d_esel,
                                                        n_esel, RT, MT, Bpad / 32, ngr, NS, p->d_pref, p->d_err, sym,
                                                        S);
     } else {
-        BL_CUDA(allow_opt_in_smem(k_reduce_tc<kNB>, p->device));
         k_reduce_tc<kNB><<<grid, 32 * W, smem, s>>>(dreq, (const float *)ypart, U, n, p->X, p->L, d_esel, n_esel,
                                                     RT, MT, Bpad / 32, ngr, NS, p->d_pref, p->d_err, sym, S);
     }

@@ -266,21 +266,20 @@ __global__ void k_reduce(const ReqDev *__restrict__ reqs, const T *__restrict__ 
 
 }  // namespace
 
-int preload_fp64_kernels()
+int preload_fp64_kernels(int device)
 {
     cudaFuncAttributes fa;
-    BL_CUDA(cudaFuncGetAttributes(&fa, k_fit));
+    BL_CUDA(allow_opt_in_smem(k_fit, device));
     BL_CUDA(cudaFuncGetAttributes(&fa, k_weights));
     BL_CUDA(cudaFuncGetAttributes(&fa, k_contract<double, false>));
     BL_CUDA(cudaFuncGetAttributes(&fa, k_contract<double, true>));
     BL_CUDA(cudaFuncGetAttributes(&fa, k_reduce<double>));
-    return BLAST_OK;
+    return fx_kernels(device);
 }
 
 int launch_fit(blast_plan *p, ReqDev *dreq, int nreq, cudaStream_t s)
 {
     size_t smem = sizeof(double) * (10 * kMaxPtab + p->N);
-    BL_CUDA(allow_opt_in_smem(k_fit, p->device));
     k_fit<<<nreq, kFitThreads, smem, s>>>(dreq, p->N, p->d_kcheb_u, p->d_cos_tab);
     BL_CUDA(cudaGetLastError());
     return BLAST_OK;
@@ -297,6 +296,7 @@ int launch_weights(blast_plan *p, ReqDev *dreq, int nreq, int want32, cudaStream
 int launch_contract(blast_plan *p, ReqDev *dreq, int nreq, int prec, const int *d_esel, int n_esel,
                     void *ypart, cudaStream_t s)
 {
+    if (prec == BLAST_FP64 && p->fx_ok) return launch_contract_fx(p, dreq, nreq, d_esel, n_esel, (double *)ypart, s);
     dim3 grid(nreq, p->X, 3 * n_esel);
     const size_t sm64 = sizeof(double) * p->N, sm32 = sizeof(float) * p->N;
     if (prec == BLAST_FP64) {

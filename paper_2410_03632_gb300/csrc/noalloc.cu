@@ -83,7 +83,7 @@ int noalloc_prepare(int dev)
     if (rc) return rc;
     cudaFuncAttributes fa;
     BL_CUDA(cudaFuncGetAttributes(&fa, k_put_desc));
-    return preload_fp64_kernels();
+    return preload_fp64_kernels(dev);
 }
 
 extern "C" int blast_cl_noalloc(blast_plan *p, const blast_request *r, double *cl_out, void *stream)

@@ -162,10 +162,11 @@ template <class T> static int dev_copy(T **dst, const std::vector<T> &src)
 static void plan_free_device(blast_plan *p)
 {
     void *bufs[] = {p->d_chi, p->d_wchi, p->d_wR, p->d_kcheb_u, p->d_cos_tab, p->d_pref, p->d_env, p->d_ell,
-                    p->T64, p->T32, p->Tsl, p->scT};
+                    p->T64, p->T32, p->Tsl, p->scT, p->colexp, p->d_slab};
     for (void *b : bufs) if (b) cudaFree(b);
     p->d_chi = p->d_wchi = p->d_wR = p->d_kcheb_u = p->d_cos_tab = p->d_pref = p->d_env = nullptr;
     p->d_ell = nullptr;
+    p->colexp = nullptr; p->d_slab = nullptr;
     p->T64 = nullptr; p->T32 = nullptr; p->Tsl = nullptr; p->scT = nullptr;
     if (p->h_err) cudaFreeHost(p->h_err);
     p->h_err = p->d_err = nullptr;
@@ -327,7 +328,14 @@ extern "C" int blast_plan_create(const blast_plan_desc *d, blast_plan **out)
         delete p;
         return BLAST_EDEVICE;
     }
-    if ((rc = noalloc_prepare(p->device))) {
+    if (cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&p->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device) != cudaSuccess) {
+        cudaGetLastError();
+        plan_free_device(p);
+        delete p;
+        return BLAST_EDEVICE;
+    }
+    if ((rc = noalloc_prepare(p->device)) || (rc = tc_kernels(p->device)) || (rc = limber_kernels(p->device))) {
         plan_free_device(p);
         delete p;
         return rc;

@@ -370,14 +370,15 @@ int launch_basis(blast_plan *p, cudaStream_t s)
 int launch_basis_convert(blast_plan *p, unsigned mask, cudaStream_t s)
 {
     size_t n = (size_t)3 * p->L * p->N * p->Q;
+    int rc = fx_prepare(p, s);
+    if (rc) return rc;
     if ((mask & BLAST_BASIS_FP32) && p->T32) {
         k_basis_to_f32<<<152 * 8, 256, 0, s>>>(p->T64, p->T32, n);
         BL_CUDA(cudaGetLastError());
         p->have32 = true;
     }
     if ((mask & BLAST_BASIS_BF16S) && p->Tsl) {
-        int rc = launch_basis_slices(p, s);
-        if (rc) return rc;
+        if ((rc = launch_basis_slices(p, s))) return rc;
         p->havebf = true;
     }
     return BLAST_OK;
