@@ -172,6 +172,9 @@ int fx_prepare(blast_plan *p, cudaStream_t s);
 int launch_contract_fx(blast_plan *p, const ReqDev *dreq, int n, const int *d_esel, int n_esel, double *Y,
                        cudaStream_t s);
 int fx_kernels(int device);
+// FP32 contraction (contract_f32.cu), same partials in FP32.
+int launch_contract_f32(blast_plan *p, const ReqDev *dreq, int n, const int *d_esel, int n_esel, float *Y,
+                        cudaStream_t s);
 int launch_reduce(blast_plan *p, ReqDev *dreq, int nreq, int prec, const int *d_esel, int n_esel,
                   const void *ypart, cudaStream_t s);
 int launch_contract_tc(blast_plan *p, ReqDev *dreq, int nreq, const int *d_esel, int n_esel,

@@ -1,0 +1,173 @@
+// FP32 contraction (a) with the R sum of quadrature (b), on CUDA cores:
+//
+//   w_b(q) = sum_n a_b[n] T~[t][l][n][q],  Y_b(t, l, a, j) = sum_r V_bj(a, r) w_b(a n_R + r).
+//
+// A block of two warps owns one chi node of one (type, ell) and BB
+// cosmologies.  A thread keeps w of NQ R nodes for all of them, so a basis
+// value is loaded once per BB multiply-adds and a coefficient (a broadcast from
+// shared memory) once per NQ, and the sums over lanes are halved in width at
+// every step: BB values cost BB shuffles, not 5 BB.  Blocks run over the
+// cosmology groups first (they share the basis tile in L2), then over (type,
+// ell) (they share the weights), then over chi nodes.
+//
+// Order of the sums: n ascending, then the R nodes of a lane (r = lane + 32 v +
+// 128 k, v = 0..3) in ascending k, the lanes of each v in the tree 16, 8, 4, 2,
+// 1, and v = 0..3 in turn.  It depends on nothing but n_R, so a cosmology's
+// bits are the same in every batch and for every BB and NQ.
+//
+// Bound by issue: multiply-adds, and the loads and shuffles between them.  48
+// cosmologies (64 ells, 128 x 128 nodes, order 64, 5+5 tracers) take 1.2 ms;
+// one block per cosmology and node, which re-read the basis from L2 for each
+// and shuffled five times per tracer, took 19 ms.
+#include "blast_internal.h"
+
+namespace {
+
+constexpr int kThreads = 64;
+
+// Sum over the 32 lanes of each of the BB values x[0..BB): the width halves
+// while more than one value is left.  Returns the sum of value `mine`.
+template <int BB>
+__device__ __forceinline__ float lane_sums(float (&x)[BB], int lane, int &mine)
+{
+    mine = 0;
+    int o = 16;
+#pragma unroll
+    for (int wdt = BB / 2; wdt >= 1; wdt /= 2, o /= 2) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < BB / 2; k++) {
+            if (k >= wdt) break;
+            const float keep = up ? x[k + wdt] : x[k], send = up ? x[k] : x[k + wdt];
+            x[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+        if (up) mine += wdt;
+    }
+    for (; o >= 1; o /= 2) x[0] += __shfl_xor_sync(0xffffffffu, x[0], o);
+    return x[0];
+}
+
+template <int BB, int NQ>
+__global__ void __launch_bounds__(kThreads)
+k_contract_f32(const ReqDev *__restrict__ reqs, int n, const float *__restrict__ basis, int L, int N, int X, int Rn,
+               const int *__restrict__ esel, int n_esel, int MT, int sym, int ngr, float *__restrict__ Y)
+{
+    extern __shared__ float4 sm4[];
+    float *as = reinterpret_cast<float *>(sm4);  // [N][BB]
+    float *red = as + (size_t)N * BB;            // [tracer][v][BB]
+    __shared__ const float *sV[BB];
+    __shared__ int sB[BB];
+    const int g = blockIdx.x % ngr, rest = blockIdx.x / ngr;
+    const int a = rest / (3 * n_esel), tl = rest - a * 3 * n_esel;
+    const int t = tl / n_esel, es = tl - t * n_esel, e = esel[es];
+    const int b0 = g * BB, nb = min(BB, n - b0), Q = X * Rn;
+    const int tid = threadIdx.x, lane = tid & 31, pw = tid >> 5;
+    const bool both = sym && t == 1;
+    for (int i = tid; i < N * BB; i += kThreads) {
+        const int b = i % BB;
+        as[i] = b < nb ? reqs[b0 + b].a32[i / BB] : 0.f;
+    }
+    if (tid < BB) {
+        const bool live = tid < nb;
+        const int ng = live ? reqs[b0 + tid].n_clust : 0, ns = live ? reqs[b0 + tid].n_lens : 0;
+        sB[tid] = t == 0 ? ng : both ? ng + ns : ns;
+        sV[tid] = live ? reqs[b0 + tid].V32 + (size_t)(t == 0 || both ? 0 : ng) * Q + (size_t)a * Rn : nullptr;
+    }
+    __syncthreads();
+    int most = 0;
+#pragma unroll
+    for (int b = 0; b < BB; b++) most = max(most, sB[b]);
+
+    float w[BB][NQ];
+#pragma unroll
+    for (int b = 0; b < BB; b++)
+#pragma unroll
+        for (int i = 0; i < NQ; i++) w[b][i] = 0.f;
+    const float *Tb = basis + ((size_t)t * L + e) * N * Q + (size_t)a * Rn;
+    int at[NQ];  // past the end: the last node again, not used
+#pragma unroll
+    for (int i = 0; i < NQ; i++) at[i] = min(32 * (pw + 2 * i) + lane, Rn - 1);
+#pragma unroll 4
+    for (int k = 0; k < N; k++) {
+        float tv[NQ], av[BB];
+#pragma unroll
+        for (int i = 0; i < NQ; i++) tv[i] = __ldg(Tb + (size_t)k * Q + at[i]);
+        if constexpr (BB % 4 == 0) {
+#pragma unroll
+            for (int b = 0; b < BB; b += 4) {
+                const float4 v = *reinterpret_cast<const float4 *>(as + (size_t)k * BB + b);
+                av[b] = v.x; av[b + 1] = v.y; av[b + 2] = v.z; av[b + 3] = v.w;
+            }
+        } else {
+#pragma unroll
+            for (int b = 0; b < BB; b++) av[b] = as[(size_t)k * BB + b];
+        }
+#pragma unroll
+        for (int b = 0; b < BB; b++)
+#pragma unroll
+            for (int i = 0; i < NQ; i++) w[b][i] = fmaf(av[b], tv[i], w[b][i]);
+    }
+    for (int j = 0; j < most; j++) {
+        float v[BB][NQ];
+#pragma unroll
+        for (int b = 0; b < BB; b++)
+#pragma unroll
+            for (int i = 0; i < NQ; i++) v[b][i] = j < sB[b] ? __ldg(sV[b] + (size_t)j * Q + at[i]) : 0.f;
+#pragma unroll
+        for (int p = 0; p < 2 && p < NQ; p++) {
+            const int vw = pw + 2 * p;
+            if (32 * vw >= Rn) break;
+            float part[BB];
+#pragma unroll
+            for (int b = 0; b < BB; b++) {
+                part[b] = 0.f;
+#pragma unroll
+                for (int i = p; i < NQ; i += 2)
+                    if (32 * (pw + 2 * i) + lane < Rn) part[b] = fmaf(v[b][i], w[b][i], part[b]);
+            }
+            int mine;
+            const float s = lane_sums<BB>(part, lane, mine);
+            if (lane % (32 / BB) == 0) red[(j * 4 + vw) * BB + mine] = s;
+        }
+    }
+    __syncthreads();
+    const int nv = min(4, (Rn + 31) / 32);
+    for (int i = tid; i < most * BB; i += kThreads) {
+        const int j = i / BB, b = i % BB;
+        if (j >= sB[b]) continue;
+        float s = 0.f;
+        for (int v = 0; v < nv; v++) s += red[(j * 4 + v) * BB + b];
+        Y[((((size_t)(b0 + b) * 3 + t) * n_esel + es) * X + a) * MT + j] = s;
+    }
+}
+
+template <int BB, int NQ>
+int launch(blast_plan *p, const ReqDev *dreq, int n, const int *d_esel, int n_esel, float *Y, cudaStream_t s)
+{
+    const int ngr = (n + BB - 1) / BB;
+    const size_t smem = sizeof(float) * ((size_t)p->N * BB + (size_t)p->max_tr * 4 * BB);  // at most 16 KB
+    k_contract_f32<BB, NQ><<<(unsigned)ngr * p->X * 3 * n_esel, kThreads, smem, s>>>(
+        dreq, n, p->T32, p->L, p->N, p->X, p->Rn, d_esel, n_esel, p->max_tr, p->r_form == 1, ngr, Y);
+    BL_CUDA(cudaGetLastError());
+    return BLAST_OK;
+}
+
+}  // namespace
+
+// NQ R nodes a thread (64 NQ >= n_R); BB as many cosmologies as leave 32
+// accumulators, 4 for two to eight cosmologies (16 would multiply for empty
+// places), 1 for one.
+int launch_contract_f32(blast_plan *p, const ReqDev *dreq, int n, const int *d_esel, int n_esel, float *Y,
+                        cudaStream_t s)
+{
+    const int nq = (p->Rn + 63) / 64;
+    if (nq <= 2)
+        return n == 1   ? launch<1, 2>(p, dreq, n, d_esel, n_esel, Y, s)
+               : n <= 8 ? launch<4, 2>(p, dreq, n, d_esel, n_esel, Y, s)
+                        : launch<16, 2>(p, dreq, n, d_esel, n_esel, Y, s);
+    if (nq <= 4)
+        return n == 1   ? launch<1, 4>(p, dreq, n, d_esel, n_esel, Y, s)
+               : n <= 4 ? launch<4, 4>(p, dreq, n, d_esel, n_esel, Y, s)
+                        : launch<8, 4>(p, dreq, n, d_esel, n_esel, Y, s);
+    return n == 1 ? launch<1, 8>(p, dreq, n, d_esel, n_esel, Y, s) : launch<4, 8>(p, dreq, n, d_esel, n_esel, Y, s);
+}

@@ -167,45 +167,40 @@ __global__ void k_weights(ReqDev *reqs, int X, int Rn, const double *__restrict_
 }
 
 // ---------------------------------------------------------------------------
-// (a) + first half of (b) on CUDA cores.  One CTA per (request, chi node a,
+// (a) + first half of (b) in FP64 multiply-adds, for basis tables that the
+// digits of the tensor-core contraction do not hold.  One CTA per (request, chi node a,
 // type t and selected ell); each thread owns R nodes r = tid, tid + blockDim...
 //   w = sum_n a_n T[t][e][n][a n_R + r],  Y[j] = sum_r V_j(a, r) w
 // reduced over r with warp shuffles, written to Y[b][t][es][a][j].
 // ---------------------------------------------------------------------------
-template <class T> struct Prec;
-template <> struct Prec<double> { static __device__ const double *a(const ReqDev &r) { return r.a64; }
-                                  static __device__ const double *V(const ReqDev &r) { return r.V64; } };
-template <> struct Prec<float> { static __device__ const float *a(const ReqDev &r) { return r.a32; }
-                                 static __device__ const float *V(const ReqDev &r) { return r.V32; } };
-
 // SYM (the symmetrised form of App. A): the gs list holds both kinds, so that
 // the reduction can add K^B_j(chi) sum_r V^A_i w to K^A_i(chi) sum_r V^B_j w.
-template <class T, bool SYM>
+template <bool SYM>
 __global__ void __launch_bounds__(128)
-k_contract(const ReqDev *__restrict__ reqs, const T *__restrict__ basis, int L, int N, int X, int Rn,
-           const int *__restrict__ esel, int n_esel, int MT, T *__restrict__ Y)
+k_contract(const ReqDev *__restrict__ reqs, const double *__restrict__ basis, int L, int N, int X, int Rn,
+           const int *__restrict__ esel, int n_esel, int MT, double *__restrict__ Y)
 {
     constexpr int MJ = SYM ? BLAST_MAX_TRACERS : BLAST_MAX_TRACERS / 2;  // tracers of one list
     extern __shared__ unsigned char smraw[];
-    T *as = reinterpret_cast<T *>(smraw);  // [N]
-    __shared__ T red[4][BLAST_MAX_TRACERS];
+    double *as = reinterpret_cast<double *>(smraw);  // [N]
+    __shared__ double red[4][BLAST_MAX_TRACERS];
     const int b = blockIdx.x, a = blockIdx.y;
     const int t = blockIdx.z / n_esel, es = blockIdx.z % n_esel;
     const int e = esel[es];
     const ReqDev &rq = reqs[b];
     const int ng = rq.n_clust, ns = rq.n_lens;
     const int nB = (t == 0) ? ng : (SYM && t == 1) ? ng + ns : ns, offB = (t == 0 || (SYM && t == 1)) ? 0 : ng;
-    const T *acoef = Prec<T>::a(rq);
+    const double *acoef = rq.a64;
     for (int n = threadIdx.x; n < N; n += blockDim.x) as[n] = acoef[n];
     __syncthreads();
     const int Q = X * Rn;
-    const T *Tb = basis + ((size_t)t * L + e) * N * Q + (size_t)a * Rn;
-    const T *V = Prec<T>::V(rq) + (size_t)offB * Q + (size_t)a * Rn;
-    T part[MJ];
+    const double *Tb = basis + ((size_t)t * L + e) * N * Q + (size_t)a * Rn;
+    const double *V = rq.V64 + (size_t)offB * Q + (size_t)a * Rn;
+    double part[MJ];
 #pragma unroll
     for (int j = 0; j < MJ; j++) part[j] = 0;
     for (int r = threadIdx.x; r < Rn; r += blockDim.x) {
-        T w = 0;
+        double w = 0;
         for (int n = 0; n < N; n++) w = fma(as[n], Tb[(size_t)n * Q + r], w);
 #pragma unroll
         for (int j = 0; j < MJ; j++)
@@ -215,13 +210,13 @@ k_contract(const ReqDev *__restrict__ reqs, const T *__restrict__ basis, int L, 
 #pragma unroll
     for (int j = 0; j < MJ; j++) {
         if (j >= nB) break;
-        T v = part[j];
+        double v = part[j];
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) red[warp][j] = v;
     }
     __syncthreads();
     if (threadIdx.x < nB) {
-        T s = 0;
+        double s = 0;
         for (int w = 0; w < (int)(blockDim.x >> 5); w++) s += red[w][threadIdx.x];
         Y[((((size_t)b * 3 + t) * n_esel + es) * X + a) * MT + threadIdx.x] = s;
     }
@@ -271,8 +266,8 @@ int preload_fp64_kernels(int device)
     cudaFuncAttributes fa;
     BL_CUDA(allow_opt_in_smem(k_fit, device));
     BL_CUDA(cudaFuncGetAttributes(&fa, k_weights));
-    BL_CUDA(cudaFuncGetAttributes(&fa, k_contract<double, false>));
-    BL_CUDA(cudaFuncGetAttributes(&fa, k_contract<double, true>));
+    BL_CUDA(cudaFuncGetAttributes(&fa, k_contract<false>));
+    BL_CUDA(cudaFuncGetAttributes(&fa, k_contract<true>));
     BL_CUDA(cudaFuncGetAttributes(&fa, k_reduce<double>));
     return fx_kernels(device);
 }
@@ -297,23 +292,11 @@ int launch_contract(blast_plan *p, ReqDev *dreq, int nreq, int prec, const int *
                     void *ypart, cudaStream_t s)
 {
     if (prec == BLAST_FP64 && p->fx_ok) return launch_contract_fx(p, dreq, nreq, d_esel, n_esel, (double *)ypart, s);
+    if (prec == BLAST_FP32) return launch_contract_f32(p, dreq, nreq, d_esel, n_esel, (float *)ypart, s);
     dim3 grid(nreq, p->X, 3 * n_esel);
-    const size_t sm64 = sizeof(double) * p->N, sm32 = sizeof(float) * p->N;
-    if (prec == BLAST_FP64) {
-        if (p->r_form == 1)
-            k_contract<double, true><<<grid, 128, sm64, s>>>(dreq, p->T64, p->L, p->N, p->X, p->Rn, d_esel, n_esel,
-                                                             p->max_tr, (double *)ypart);
-        else
-            k_contract<double, false><<<grid, 128, sm64, s>>>(dreq, p->T64, p->L, p->N, p->X, p->Rn, d_esel, n_esel,
-                                                              p->max_tr, (double *)ypart);
-    } else {
-        if (p->r_form == 1)
-            k_contract<float, true><<<grid, 128, sm32, s>>>(dreq, p->T32, p->L, p->N, p->X, p->Rn, d_esel, n_esel,
-                                                            p->max_tr, (float *)ypart);
-        else
-            k_contract<float, false><<<grid, 128, sm32, s>>>(dreq, p->T32, p->L, p->N, p->X, p->Rn, d_esel, n_esel,
-                                                             p->max_tr, (float *)ypart);
-    }
+    const size_t smem = sizeof(double) * p->N;
+    (p->r_form == 1 ? k_contract<true> : k_contract<false>)<<<grid, 128, smem, s>>>(
+        dreq, p->T64, p->L, p->N, p->X, p->Rn, d_esel, n_esel, p->max_tr, (double *)ypart);
     BL_CUDA(cudaGetLastError());
     return BLAST_OK;
 }
