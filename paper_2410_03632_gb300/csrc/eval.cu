@@ -20,11 +20,6 @@ namespace {
 constexpr int kFitThreads = 256;
 constexpr int kMaxPtab = 1024;
 
-__device__ __forceinline__ int npairs_dev(int ng, int ns)
-{
-    return ng * (ng + 1) / 2 + ng * ns + ns * (ns + 1) / 2;
-}
-
 // Pair p of a (ng, ns) tracer set -> type t (0 gg, 1 gs, 2 ss), A-side tracer
 // row i and B-side tracer row j (both as rows of the request's kernel arrays).
 __device__ __forceinline__ void pair_decode(int p, int ng, int ns, int &t, int &ia, int &jb, int &jloc)
@@ -224,38 +219,47 @@ k_contract(const ReqDev *__restrict__ reqs, const double *__restrict__ basis, in
 
 // ---------------------------------------------------------------------------
 // Second half of (b): C_ij(l) = N_AB(l) sum_a U_i(a) Y[t][es][a][j], summed in
-// FP64, scattered to the request's output columns.
-// ---------------------------------------------------------------------------
+// FP64, scattered to the request's output columns.  A block owns one (request,
+// type, selected ell), eight lanes a pair: lane c sums a = c, c + 8, .. and the
+// lanes meet in a tree, so the chain of a pair is X / 8 long (a thread per pair
+// waited for X loads and multiply-adds in turn: 36 us for one cosmology of
+// 5+5 tracers on 128 chi nodes and 64 ells, 88 us for 10+10 on 256 and 32).
+//
 // sym: C_ij also gets N_AB(l) sum_a U_j(a) Y[t][es][a][i] (both kernel orders
 // of the symmetrised form, App. A); list positions are tracer rows minus the
 // list's first row.
+// ---------------------------------------------------------------------------
+constexpr int kRedThreads = 256, kRedLanes = 8;
+
 template <class T>
-__global__ void k_reduce(const ReqDev *__restrict__ reqs, const T *__restrict__ Y, int X, int L,
-                         const int *__restrict__ esel, int n_esel, int MT, const double *__restrict__ pref, int sym)
+__global__ void __launch_bounds__(kRedThreads)
+k_reduce(const ReqDev *__restrict__ reqs, const T *__restrict__ Y, int X, int L, const int *__restrict__ esel,
+         int n_esel, int MT, const double *__restrict__ pref, int sym)
 {
-    const int b = blockIdx.y;
+    const int es = blockIdx.x, t = blockIdx.y, b = blockIdx.z, e = esel[es];
     const ReqDev &rq = reqs[b];
-    const int ng = rq.n_clust, ns = rq.n_lens, P = npairs_dev(ng, ns);
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < P * n_esel; idx += gridDim.x * blockDim.x) {
-        const int p = idx / n_esel, es = idx % n_esel, e = esel[es];
-        const int col = rq.e_out[e];
-        if (col < 0) continue;
-        int t, ia, jb, jloc;
-        pair_decode(p, ng, ns, t, ia, jb, jloc);
-        const double *U = rq.U64 + (size_t)ia * X;
-        const int first = (t == 0 || (sym && t == 1)) ? 0 : ng;  // first tracer row of the type's list
-        const T *Yb = Y + (((size_t)b * 3 + t) * n_esel + es) * (size_t)X * MT;
-        const T *Yp = Yb + (jb - first);
+    const int col = rq.e_out[e];
+    if (col < 0) return;
+    const int ng = rq.n_clust, ns = rq.n_lens, ngg = ng * (ng + 1) / 2, ngs = ng * ns;
+    const int p0 = t == 0 ? 0 : t == 1 ? ngg : ngg + ngs;
+    const int np = t == 0 ? ngg : t == 1 ? ngs : ns * (ns + 1) / 2;
+    const int first = (t == 0 || (sym && t == 1)) ? 0 : ng;  // first tracer row of the type's list
+    const T *Yb = Y + (((size_t)b * 3 + t) * n_esel + es) * (size_t)X * MT;
+    const int c = threadIdx.x % kRedLanes;
+    const unsigned mask = 0xffu << (threadIdx.x & 24);
+    auto dot = [&](const double *U, const T *y) {
         double s = 0.0;
-        for (int a = 0; a < X; a++) s = fma(U[a], (double)Yp[(size_t)a * MT], s);
-        if (sym) {
-            const double *Uj = rq.U64 + (size_t)jb * X;
-            const T *Yi = Yb + (ia - first);
-            for (int a = 0; a < X; a++) s = fma(Uj[a], (double)Yi[(size_t)a * MT], s);
-        }
-        double out = pref[t * L + e] * s;
-        if (rq.status) out = nan("");
-        rq.cl[(size_t)p * rq.n_sel + col] = out;
+#pragma unroll 8
+        for (int a = c; a < X; a += kRedLanes) s = fma(U[a], (double)y[(size_t)a * MT], s);
+        return s;
+    };
+    for (int p = threadIdx.x / kRedLanes; p < np; p += kRedThreads / kRedLanes) {
+        int tt, ia, jb, jloc;
+        pair_decode(p0 + p, ng, ns, tt, ia, jb, jloc);
+        double s = dot(rq.U64 + (size_t)ia * X, Yb + (jb - first));
+        if (sym) s += dot(rq.U64 + (size_t)jb * X, Yb + (ia - first));
+        for (int o = kRedLanes / 2; o; o /= 2) s += __shfl_xor_sync(mask, s, o);
+        if (c == 0) rq.cl[(size_t)(p0 + p) * rq.n_sel + col] = rq.status ? nan("") : pref[t * L + e] * s;
     }
 }
 
@@ -304,15 +308,17 @@ int launch_contract(blast_plan *p, ReqDev *dreq, int nreq, int prec, const int *
 int launch_reduce(blast_plan *p, ReqDev *dreq, int nreq, int prec, const int *d_esel, int n_esel,
                   const void *ypart, cudaStream_t s)
 {
-    int pmax = blast_npairs(p->max_clust, p->max_lens);
-    dim3 grid((pmax * n_esel + 127) / 128, nreq);
-    if (prec == BLAST_FP64)
-        k_reduce<double><<<grid, 128, 0, s>>>(dreq, (const double *)ypart, p->X, p->L, d_esel, n_esel, p->max_tr,
-                                              p->d_pref, p->r_form);
-    else
-        k_reduce<float><<<grid, 128, 0, s>>>(dreq, (const float *)ypart, p->X, p->L, d_esel, n_esel, p->max_tr,
-                                             p->d_pref, p->r_form);
-    BL_CUDA(cudaGetLastError());
+    for (int b0 = 0; b0 < nreq; b0 += 65535) {  // the largest grid in z
+        const dim3 grid(n_esel, 3, nreq - b0 < 65535 ? nreq - b0 : 65535);
+        const size_t y0 = (size_t)b0 * 3 * n_esel * p->X * p->max_tr;
+        if (prec == BLAST_FP64)
+            k_reduce<double><<<grid, kRedThreads, 0, s>>>(dreq + b0, (const double *)ypart + y0, p->X, p->L, d_esel,
+                                                          n_esel, p->max_tr, p->d_pref, p->r_form);
+        else
+            k_reduce<float><<<grid, kRedThreads, 0, s>>>(dreq + b0, (const float *)ypart + y0, p->X, p->L, d_esel,
+                                                         n_esel, p->max_tr, p->d_pref, p->r_form);
+        BL_CUDA(cudaGetLastError());
+    }
     return BLAST_OK;
 }
 
