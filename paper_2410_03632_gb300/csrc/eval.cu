@@ -49,12 +49,14 @@ k_fit(ReqDev *reqs, int N, const double *__restrict__ node_u, const double *__re
     const int n = rq.n_ptab;
     extern __shared__ double sh[];
     double *u = sh, *v = u + n;
-    double *A0 = v + n, *B0 = A0 + n, *C0 = B0 + n, *D0 = C0 + n;
-    double *A1 = D0 + n, *B1 = A1 + n, *C1 = B1 + n, *D1 = C1 + n;
+    double *A0 = v + n, *C0 = A0 + n, *D0 = C0 + n;
+    double *A1 = D0 + n, *C1 = A1 + n, *D1 = C1 + n;
     double *Pn = D1 + n;  // [N]
+    double *ct = Pn + N;  // [4N] cos(pi p / 2N)
     __shared__ int bad;
     const int tid = threadIdx.x;
     if (tid == 0) bad = 0;
+    for (int i = tid; i < 4 * N; i += blockDim.x) ct[i] = cos_tab[i];
     __syncthreads();
     for (int i = tid; i < n; i += blockDim.x) {
         double k = rq.k_tab[i], P = rq.p_tab[i];
@@ -65,36 +67,43 @@ k_fit(ReqDev *reqs, int N, const double *__restrict__ node_u, const double *__re
     __syncthreads();
     for (int i = tid + 1; i < n; i += blockDim.x)
         if (!(u[i] > u[i - 1])) bad = 1;
-    // tridiagonal system for the spline second derivatives M_i, M_0 = M_{n-1} = 0
+    // tridiagonal system for the spline second derivatives M_i, M_0 = M_{n-1} = 0,
+    // every row divided by its diagonal: M_i + A_i M_{i-1} + C_i M_{i+1} = D_i
     for (int i = tid; i < n; i += blockDim.x) {
-        if (i == 0 || i == n - 1) { A0[i] = 0.0; B0[i] = 1.0; C0[i] = 0.0; D0[i] = 0.0; continue; }
-        double hl = u[i] - u[i - 1], hr = u[i + 1] - u[i];
-        A0[i] = hl; B0[i] = 2.0 * (hl + hr); C0[i] = hr;
-        D0[i] = 6.0 * ((v[i + 1] - v[i]) / hr - (v[i] - v[i - 1]) / hl);
+        if (i == 0 || i == n - 1) { A0[i] = 0.0; C0[i] = 0.0; D0[i] = 0.0; continue; }
+        const double hl = u[i] - u[i - 1], hr = u[i + 1] - u[i], r = 0.5 / (hl + hr);
+        A0[i] = hl * r; C0[i] = hr * r;
+        D0[i] = 6.0 * r * ((v[i + 1] - v[i]) / hr - (v[i] - v[i - 1]) / hl);
     }
     __syncthreads();
-    // parallel cyclic reduction: after ceil(log2 n) sweeps every row is decoupled
-    double *a = A0, *b = B0, *c = C0, *d = D0, *a2 = A1, *b2 = B1, *c2 = C1, *d2 = D1;
+    // Parallel cyclic reduction: each sweep couples rows twice as far apart and
+    // squares the couplings (at most 1/2 each at the start: the matrix is
+    // diagonally dominant), so a row is decoupled after ceil(log2 n) sweeps, or
+    // earlier, once no coupling is above 2^-64: what is left out then is below
+    // 2^-63 of the largest M.  One reciprocal a row and sweep.
+    double *a = A0, *c = C0, *d = D0, *a2 = A1, *c2 = C1, *d2 = D1;
     for (int s = 1; s < n; s <<= 1) {
+        int coupled = 0;
         for (int i = tid; i < n; i += blockDim.x) {
-            int im = i - s, ip = i + s;
-            double al = (im >= 0) ? -a[i] / b[im] : 0.0;
-            double ga = (ip < n) ? -c[i] / b[ip] : 0.0;
-            a2[i] = (im >= 0) ? al * a[im] : 0.0;
-            c2[i] = (ip < n) ? ga * c[ip] : 0.0;
-            b2[i] = b[i] + ((im >= 0) ? al * c[im] : 0.0) + ((ip < n) ? ga * a[ip] : 0.0);
-            d2[i] = d[i] + ((im >= 0) ? al * d[im] : 0.0) + ((ip < n) ? ga * d[ip] : 0.0);
+            const int im = i - s, ip = i + s;
+            const double al = im >= 0 ? a[i] : 0.0, ga = ip < n ? c[i] : 0.0;
+            const double am = im >= 0 ? a[im] : 0.0, cm = im >= 0 ? c[im] : 0.0, dm = im >= 0 ? d[im] : 0.0;
+            const double ap = ip < n ? a[ip] : 0.0, cp = ip < n ? c[ip] : 0.0, dp = ip < n ? d[ip] : 0.0;
+            const double r = 1.0 / fma(-ga, ap, fma(-al, cm, 1.0));
+            const double an = -al * am * r, cn = -ga * cp * r;
+            a2[i] = an;
+            c2[i] = cn;
+            d2[i] = fma(-ga, dp, fma(-al, dm, d[i])) * r;
+            coupled |= fabs(an) > 0x1p-64 || fabs(cn) > 0x1p-64;
         }
-        __syncthreads();
+        coupled = __syncthreads_or(coupled);
         double *t;
-        t = a; a = a2; a2 = t; t = b; b = b2; b2 = t; t = c; c = c2; c2 = t; t = d; d = d2; d2 = t;
+        t = a; a = a2; a2 = t; t = c; c = c2; c2 = t; t = d; d = d2; d2 = t;
+        if (!coupled) break;
     }
-    double *M = a2;  // reuse a free buffer
-    for (int i = tid; i < n; i += blockDim.x) {
-        M[i] = d[i] / b[i];
-        if (rq.spM) rq.spM[i] = M[i];  // kept for the Limber terms
-    }
-    __syncthreads();
+    const double *M = d;
+    if (rq.spM)
+        for (int i = tid; i < n; i += blockDim.x) rq.spM[i] = M[i];  // kept for the Limber terms
     // spline at the Chebyshev nodes, then exp
     for (int j = tid; j < N; j += blockDim.x) {
         double x = node_u[j];
@@ -106,19 +115,29 @@ k_fit(ReqDev *reqs, int N, const double *__restrict__ node_u, const double *__re
         Pn[j] = exp(val);
     }
     __syncthreads();
-    // a_n = (c_n / N) sum_j P_j cos(n (2j+1) pi / 2N), c_0 = 1, c_n = 2
-    for (int nn = tid; nn < N; nn += blockDim.x) {
+    // a_n = (c_n / N) sum_j P_j cos(n (2j+1) pi / 2N), c_0 = 1, c_n = 2: four
+    // lanes a coefficient, lane c sums j = c, c + 4, ..
+    const int c4 = tid & 3;
+    for (int n0 = 0; n0 < N; n0 += blockDim.x / 4) {
+        const int nn = n0 + tid / 4;
         double acc = 0.0;
-        int idx = nn, step = 2 * nn, mod = 4 * N;
-        for (int j = 0; j < N; j++) {
-            acc = fma(Pn[j], cos_tab[idx], acc);
-            idx += step;
-            if (idx >= mod) idx -= mod;
+        if (nn < N) {
+            const int mod = 4 * N, step = (8 * nn) % mod;
+            int idx = nn * (2 * c4 + 1) % mod;
+            for (int j = c4; j < N; j += 4) {
+                acc = fma(Pn[j], ct[idx], acc);
+                idx += step;
+                if (idx >= mod) idx -= mod;
+            }
         }
-        double an = (nn == 0 ? 1.0 : 2.0) * acc / (double)N;
-        if (bad) an = nan("");
-        rq.a64[nn] = an;
-        rq.a32[nn] = (float)an;
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        if (nn < N && c4 == 0) {
+            double an = (nn == 0 ? 1.0 : 2.0) * acc / (double)N;
+            if (bad) an = nan("");
+            rq.a64[nn] = an;
+            rq.a32[nn] = (float)an;
+        }
     }
     if (tid == 0 && bad) rq.status = BLAST_EINVAL;
 }
@@ -278,7 +297,7 @@ int preload_fp64_kernels(int device)
 
 int launch_fit(blast_plan *p, ReqDev *dreq, int nreq, cudaStream_t s)
 {
-    size_t smem = sizeof(double) * (10 * kMaxPtab + p->N);
+    size_t smem = sizeof(double) * (8 * kMaxPtab + 5 * (size_t)p->N);
     k_fit<<<nreq, kFitThreads, smem, s>>>(dreq, p->N, p->d_kcheb_u, p->d_cos_tab);
     BL_CUDA(cudaGetLastError());
     return BLAST_OK;
