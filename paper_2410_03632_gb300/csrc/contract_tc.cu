@@ -28,19 +28,25 @@
 // oscillates around R = 1), so it runs on unevaluated pairs: exact products
 // (FMA), two products (columns two R nodes apart) added plainly, and two-sum
 // accumulation of those sums, two columns at a time in packed FP32 pairs; the
-// pairs reach the chi sum intact.
+// (hi, lo) pairs are written per R-tile and reduced by k_reduce_tc.
 //
-// Warp roles (320 threads): warp 0 issues TMA loads of the basis slices into
-// a ring of stages, warp 1 owns TMEM and issues tcgen05.mma (A = coefficient
-// slices resident in TMEM, B = basis slices in shared memory) into two
-// accumulator buffers, warps 2..9 run the epilogue (one TMEM lane = one
-// cosmology per thread, two warps per lane quadrant with 16 columns each,
-// quadrature weights of the unit's five B-side tracers in registers, the two
-// column halves joined through shared memory at a named barrier).  A work unit
-// is (cosmology tile of 128, group of five B-side tracers, 32-node q tile);
-// plans with up to ten tracers per kind run two groups as separate units.
+// Warp-specialised persistent CTAs: a TMA producer, an MMA issuer per accumulator
+// buffer, twelve epilogue warps (one cosmology per thread, three warps per TMEM
+// lane quadrant taking the tiles in turn, quadrature weights of the unit's five
+// B-side tracers in shared memory).  A work unit is (cosmology tile of 128,
+// group of five B-side tracers, 32-node q tile); plans with up to ten tracers
+// per kind run two groups as separate units.
 // Every mbarrier wait is bounded; on timeout the kernel records an error code
 // in host-mapped memory and exits after its copies and MMAs in flight complete.
+//
+// What bounds it: at order 64 the FP32 pipe (a basis tile of 128 x 32 takes 704
+// packed instructions, 1408 cycles, and 140 scalar ones per SM sub-partition, and
+// about 2350 cycles in all), at order 96 the MMAs as well (90 of 17 to 40 cycles).
+// 256 cosmologies (64 ells, 128 x 128 nodes, order 64, 5+5 tracers): 1.93 ms with
+// eight epilogue warps that held their weights in registers, took half a tile
+// each, met at a barrier and waited for the tile's scale from L2, and one issuer;
+// 1.60 ms so.  150 ragged cosmologies of up to 10+10 tracers (32 ells, 256 x 192
+// nodes, order 96): 6.05 ms and 5.04 ms.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -57,32 +63,35 @@ constexpr int kS = BLAST_TC_SLICES;       // slices per operand
 constexpr int kQT = 32;                   // chi-R nodes per tile (MMA N)
 constexpr int kM = 128;                   // cosmologies per tile (MMA M)
 constexpr int kKC = 64;                   // K elements per 128-byte swizzle row (one TMA box)
-constexpr int kEP = 2;                    // epilogue warps per TMEM lane quadrant
-constexpr int kThreads = 64 + 128 * kEP;  // 2 control warps + 4 kEP epilogue warps
-constexpr int kHC = kQT / kEP;            // columns per epilogue thread
-constexpr int kCS = 4;                    // columns per TMEM load step
-constexpr int kNB = 5;                    // tracers per weight group
 constexpr int kNBUF = 2;                  // TMEM accumulator buffers
+constexpr int kEW = 3;                    // epilogue warps per TMEM lane quadrant, tiles in turn
+constexpr int kEpi0 = 4;                  // first epilogue warp (warp 0 TMA, 1 and 2 MMA, 3 spare)
+constexpr int kThreads = 128 + 128 * kEW;
+constexpr int kFull = kNBUF * kEW;        // tile-complete barriers: one per buffer and epilogue warp
+constexpr int kHC = kQT / 2;              // columns summed together
+constexpr int kCS = 8;                    // columns per TMEM load step
+constexpr int kNB = 5;                    // tracers per weight group
 constexpr uint32_t kBSliceBytes = kQT * 128;  // 32 rows x 64 bf16
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kCtrlBytes = 256;          // mbarriers, TMEM address, abort flag
 constexpr uint32_t kEselBytes = 4 * BLAST_MAX_ELL;  // selected ells
+constexpr uint32_t kScBytes = 2 * 3 * 4 * BLAST_MAX_ELL;  // tile scales of a unit, two units
 
-// Compile-time shape of one kernel instance: KC 64-wide K chunks per stage
-// (1: order <= 64, 2: order <= 96).
+// Compile-time shape of one kernel instance: KC 64-wide K chunks per tile
+// (1: order <= 64, 2: order <= 96), one chunk per stage.
 // Both keep five exact TMEM levels; with two K chunks the coefficient slices
 // 0..3 fill the TMEM left beside the accumulators and slice 4 (one slice pair,
 // p = 4, q = 0, per K step) is read from shared memory.
 template <int KC> struct TcCfg {
     static constexpr int LV = 5;                            // TMEM accumulator levels
-    static constexpr int kStages = KC == 1 ? 8 : 4;
-    static constexpr uint32_t kStageBytes = KC * kS * kBSliceBytes;
+    static constexpr int kStages = KC == 1 ? 6 : 4;         // a multiple of 2 KC: see the issuers
+    static constexpr uint32_t kStageBytes = kS * kBSliceBytes;
     static constexpr uint32_t kACol = kNBUF * LV * kQT;     // TMEM column of the coefficient slices
     static constexpr int kSliceTmem = KC == 1 ? kS : kS - 1;  // coefficient slices held in TMEM
     static constexpr uint32_t kA4Bytes = KC == 1 ? 0 : KC * kM * 128;  // slice 4: [chunk][128 rows][128 B]
-    static constexpr int kYbufFloats = 2 * 4 * (kEP - 1) * kNB * 64;  // [parity][quadrant][part-1][tracer][hi, lo][lane]
-    static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kA4Bytes + kCtrlBytes + kEselBytes +
-                                    kYbufFloats * 4;
+    static constexpr uint32_t kVBytes = kNB * kQT * kM * 4;  // weights [tracer][4 columns][cosmology][4]
+    static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kA4Bytes + kVBytes + kCtrlBytes +
+                                    kEselBytes + kScBytes;
 };
 
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of
@@ -121,6 +130,14 @@ __device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint64_t ad, uint64_t b
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
         ::"r"(d_tmem), "l"(ad), "l"(bd), "r"(kIdesc), "r"(acc));
+}
+
+// Four floats from shared memory, not moved by the compiler.
+__device__ __forceinline__ float4 lds4(uint32_t addr)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+    return v;
 }
 
 // Knuth's two-sum: s + e == a + b exactly, s = fl(a + b).
@@ -301,6 +318,7 @@ struct TcArgs {
     const float *sa;     // [Bpad]
     const uint16_t *A;   // [S][Bpad][Kst] coefficient slices
     float *Y;            // [npass][n_esel][X][Bpad/32][ngr][RT][5][hi, lo][32] R-tile partial pairs
+    size_t ystep;        // floats of Y between ells
     int *err;            // host-mapped error word
     int trip;            // test hook: tile at which CTA 0 waits on a barrier nothing completes (-1 off)
 };
@@ -337,20 +355,20 @@ k_contract_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ 
     using C = TcCfg<KC>;
     constexpr int LV = C::LV;
     constexpr int kStages = C::kStages;
-    constexpr int NGB = kNB;  // B-side tracers of one unit
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte alignment for the swizzled tiles
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char *sB = smem;                                         // kStages x KC x kS x 4 KB
+    unsigned char *sB = smem;                                         // kStages x kS x 4 KB
     unsigned char *sA4 = sB + (size_t)kStages * C::kStageBytes;        // coefficient slice 4 (order > 64)
-    uint64_t *bars = (uint64_t *)(sA4 + C::kA4Bytes);                   // kCtrlBytes of control words
+    float *sV = (float *)(sA4 + C::kA4Bytes);                           // weights of the unit's tracers
+    uint64_t *bars = (uint64_t *)((unsigned char *)sV + C::kVBytes);    // kCtrlBytes of control words
     uint64_t *full = bars, *empty = bars + kStages, *aready = bars + 2 * kStages;
-    uint64_t *tfull = aready + 1, *tempty = tfull + kNBUF, *mdone = tempty + kNBUF, *a4ready = mdone + 1;
+    uint64_t *tfull = aready + 1, *tempty = tfull + kFull, *mdone = tempty + kNBUF, *a4ready = mdone + kNBUF;
     uint64_t *never = a4ready + 1;  // no thread ever arrives on it (test hook)
     uint32_t *tmem_slot = (uint32_t *)(never + 1);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     int *s_esel = (int *)((unsigned char *)bars + kCtrlBytes);         // selected ells
-    float *ybuf = (float *)((unsigned char *)s_esel + kEselBytes);     // [2][4][kEP-1][NGB][2][32] column-part hand-over
+    float *s_sc = (float *)((unsigned char *)s_esel + kEselBytes);     // [unit parity][type][ell] tile scales
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int btile = blockIdx.x % args.nbt;
@@ -360,8 +378,9 @@ k_contract_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; i++) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
         mbar_init(aready, 128);
-        for (int i = 0; i < kNBUF; i++) { mbar_init(&tfull[i], 1); mbar_init(&tempty[i], 128 * kEP); }
-        mbar_init(mdone, 1);
+        for (int i = 0; i < kFull; i++) mbar_init(&tfull[i], 1);
+        for (int i = 0; i < kNBUF; i++) mbar_init(&tempty[i], 128);
+        for (int i = 0; i < kNBUF; i++) mbar_init(&mdone[i], 1);
         mbar_init(a4ready, 1);
         mbar_init(never, 1);
         *abort_flag = 0;
@@ -388,40 +407,42 @@ k_contract_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ 
             }
             __syncwarp();
         }
-        uint32_t g = 0;
+        uint32_t k = 0;  // stages filled
         bool ok = true;
         for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
             int grp, q0;
             unit_decode(args, u, grp, q0);
-            for (int it = 0; it < n_iter_unit; it++, g++) {
-                const int st = g % kStages;
-                const uint32_t ph = (g / kStages) & 1;
-                const bool bad = *abort_flag || !mbar_wait(&empty[st], ph ^ 1, 64);
-                if (__any_sync(0xffffffffu, bad)) {
-                    if (lane == 0) { atomicExch(args.err, 1); *abort_flag = 1; }
-                    ok = false;
-                    break;
-                }
-                if (elect_one()) {
-                    const int t = pass_basis(it / args.n_esel, args.sym), e = s_esel[it % args.n_esel];
-                    const int row = (t * args.L + e) * args.Q + q0;
-                    mbar_expect_tx(&full[st], C::kStageBytes);
+            for (int it = 0; ok && it < n_iter_unit; it++) {
+                const int t = pass_basis(it / args.n_esel, args.sym), e = s_esel[it % args.n_esel];
+                const int row = (t * args.L + e) * args.Q + q0;
 #pragma unroll
-                    for (int c = 0; c < KC; c++)
-                        tma_load_3d(sB + (size_t)st * C::kStageBytes + c * kS * kBSliceBytes, &mapB, &full[st],
-                                    c * kKC, row, 0);
+                for (int c = 0; c < KC; c++, k++) {
+                    const int st = k % kStages;
+                    const bool bad = *abort_flag || !mbar_wait(&empty[st], ((k / kStages) & 1) ^ 1, 64);
+                    if (__any_sync(0xffffffffu, bad)) {
+                        if (lane == 0) { atomicExch(args.err, 1); *abort_flag = 1; }
+                        ok = false;
+                        break;
+                    }
+                    if (elect_one()) {
+                        mbar_expect_tx(&full[st], C::kStageBytes);
+                        tma_load_3d(sB + (size_t)st * C::kStageBytes, &mapB, &full[st], c * kKC, row, 0);
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
             }
         }
         // drain: every issued load has landed before the CTA may exit
-        for (uint32_t h = (g > (uint32_t)kStages ? g - kStages : 0); h < g; h++)
+        for (uint32_t h = (k > (uint32_t)kStages ? k - kStages : 0); h < k; h++)
             mbar_wait(&full[h % kStages], (h / kStages) & 1, 64);
         if (KC == 2) mbar_wait(a4ready, 0, 64);
         __syncwarp();
-    } else if (warp == 1) {
-        // ------------------------------------------------ MMA issuer (whole warp waits; each MMA is
-        // issued by one elected lane of the converged warp)
+    } else if (warp <= kNBUF) {
+        // ------------------------------------------------ MMA issuers, one per accumulator buffer, so
+        // that the tensor pipe has the next tile's MMAs queued while an issuer looks at its
+        // barriers (one issuer left it idle for about 1000 cycles a tile).  The stages are a
+        // multiple of two tiles, so each stage belongs to one issuer, which sees all its phases.
+        // The whole warp waits; each MMA is issued by one elected lane of the converged warp.
         bool ok = __all_sync(0xffffffffu, mbar_wait(aready, 0, 64) && (KC == 1 || mbar_wait(a4ready, 0, 64)));
         if (!ok && lane == 0) { atomicExch(args.err, 2); *abort_flag = 1; }  // coefficient slices in TMEM / smem
         tc_fence_after();
@@ -430,14 +451,17 @@ k_contract_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ 
         const int nk = args.Kmma / 16;        // K steps of 16
         const uint32_t a4base = __shfl_sync(0xffffffffu, smem_u32(sA4), 0);
         const uint32_t acol = args.Kmma / 2;  // TMEM columns per coefficient slice
-        uint32_t g = 0;
-        for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-            for (int it = 0; it < n_iter_unit; it++, g++) {
-                const int st = g % kStages;
-                const uint32_t ph = (g / kStages) & 1;
-                const int buf = g % kNBUF;
-                const uint32_t tph = (g / kNBUF) & 1;
-                const bool bad = *abort_flag || !mbar_wait(&full[st], ph, 64) || !mbar_wait(&tempty[buf], tph ^ 1, 64);
+        const int buf = warp - 1;
+        const uint32_t dbase = tm + buf * (LV * kQT);
+        const uint32_t n_tiles = blockIdx.x < n_units ? (n_units - 1 - blockIdx.x) / gridDim.x * n_iter_unit + n_iter_unit
+                                                      : 0;
+        int st = buf * KC;  // stage and its lap's parity
+        uint32_t ph = 0;
+        for (uint32_t g = buf; ok && g < n_tiles; g += kNBUF) {
+#pragma unroll
+            for (int c = 0; c < KC; c++, st++) {
+                const bool bad = *abort_flag || (c == 0 && !mbar_wait(&tempty[buf], ((g / kNBUF) & 1) ^ 1, 64)) ||
+                                 !mbar_wait(&full[st], ph, 64);
                 if (__any_sync(0xffffffffu, bad)) {
                     if (lane == 0) { atomicExch(args.err, 3); *abort_flag = 1; }
                     ok = false;
@@ -446,67 +470,60 @@ k_contract_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ 
                 tc_fence_after();
                 // operands: accumulator levels of this buffer, coefficient slices in
                 // TMEM, basis slice descriptors offset from this stage's first
-                const uint32_t dbase = tm + buf * (LV * kQT);
                 const uint64_t bbase = sdesc(b0 + st * C::kStageBytes);
+                const int k1 = min(nk - 4 * c, 4);
                 if (elect_one()) {
                     // Consecutive MMAs into one accumulator wait for each other, so the
                     // issue order interleaves the levels: per K step, rounds r = 0..4 of
                     // the slice pairs (p = r, q = k - r) over levels k = 4 .. 0, so that
                     // an accumulator is hit again only after the other levels had a turn.
-                    uint32_t started = 0;  // levels already written in this tile
-                    for (int kk = 0; kk < nk; kk++) {
-                        const uint32_t koff = (kk >> 2) * (kS * kBSliceBytes) + (kk & 3) * 32;
+                    // Round 0 of the tile's first K step starts every level.
+                    for (int kk = 0; kk < k1; kk++) {
 #pragma unroll
                         for (int r = 0; r < kS; r++) {
 #pragma unroll
-                            for (int k = kS - 1; k >= r; k--) {
-                                const int p = r, q = k - r;
-                                const int lev = k < LV - 1 ? k : LV - 1;
-                                const uint32_t boff = koff + q * kBSliceBytes;
+                            for (int lev = kS - 1; lev >= r; lev--) {
+                                const int p = r, q = lev - r;
+                                const uint32_t boff = q * kBSliceBytes + kk * 32;
                                 if (p < C::kSliceTmem)
-                                    umma_ts(dbase + lev * kQT, tm + C::kACol + p * acol + kk * 8,
-                                            bbase + (uint64_t)(boff >> 4), (started >> lev) & 1u);
+                                    umma_ts(dbase + lev * kQT, tm + C::kACol + p * acol + (4 * c + kk) * 8,
+                                            bbase + (uint64_t)(boff >> 4), (c | kk | r) != 0);
                                 else  // slice 4 from shared memory
                                     umma_ss(dbase + lev * kQT,
-                                            sdesc(a4base + (kk >> 2) * (kM * 128)) + (uint64_t)(((kk & 3) * 32) >> 4),
-                                            bbase + (uint64_t)(boff >> 4), (started >> lev) & 1u);
-                                started |= 1u << lev;
+                                            sdesc(a4base + c * (kM * 128)) + (uint64_t)((kk * 32) >> 4),
+                                            bbase + (uint64_t)(boff >> 4), (c | kk | r) != 0);
                             }
                         }
                     }
-                }
-                __syncwarp();
-                if (elect_one()) {
                     umma_commit(&empty[st]);
-                    umma_commit(&tfull[buf]);
+                    if (c == KC - 1) umma_commit(&tfull[g % kFull]);
                 }
                 __syncwarp();
             }
+            st += (kNBUF - 1) * KC;  // past the other issuer's stages
+            if (st >= kStages) { st -= kStages; ph ^= 1; }
         }
         // every MMA this warp issued has completed before TMEM is released
-        if (elect_one()) umma_commit(mdone);
+        if (elect_one()) umma_commit(&mdone[buf]);
         __syncwarp();
-        mbar_wait(mdone, 0, 64);
+        mbar_wait(&mdone[buf], 0, 64);
         __syncwarp();
-    } else {
-        // ------------------------------------------------ epilogue: kEP warps per TMEM lane quadrant;
-        // a thread owns one cosmology (TMEM lane) and kHC of the tile's 32 columns.
-        const int ew = warp - 2;
+    } else if (warp >= kEpi0) {
+        // ------------------------------------------------ epilogue: three warps per TMEM lane
+        // quadrant take the tiles in turn; a thread owns one cosmology (TMEM lane) and all 32
+        // columns of its tiles, so no sums are handed between threads.  A tile's levels are
+        // joined for every column first and its buffer goes back to the MMAs before the longer
+        // R sum.  Three warps with 128 registers hold that; four have 96, and a spill goes to
+        // L2 here (shared memory takes all of L1).
         const int quad = warp & 3;   // lanes 32 quad .. 32 quad + 31 are readable by this warp
-        const int part = ew >> 2;    // columns [kHC part, kHC part + kHC)
+        const int turn = (warp - kEpi0) >> 2;
         const int bl_ = quad * 32 + lane;
         const int b = btile * kM + bl_;
-        const bool valid = b < args.n;
         // a quadrant whose 32 lanes are all padding (a batch smaller than the
         // tile) only keeps the buffer hand-off in step
         const bool qlive = btile * kM + quad * 32 < args.n;
-        const ReqDev *rq = valid ? &args.reqs[b] : nullptr;
-        const int ng = valid ? rq->n_clust : 0, ns = valid ? rq->n_lens : 0;
-        const float sa = args.sa[b];
         const uint32_t lane_addr = ((uint32_t)(quad * 32)) << 16;
-        const int cb = part * kHC;
-        const int tid_e = threadIdx.x - 64;  // 0 .. 128 kEP - 1
-        if (part == 0) {
+        if (turn == 0) {
             // coefficient slices of cosmology b -> TMEM lane b, columns kACol + (Kmma/2) p ..
             const int acol = args.Kmma / 2;
 #pragma unroll 1
@@ -523,168 +540,175 @@ k_contract_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ 
             tc_fence_before();
             mbar_arrive(aready);
         }
-        // Every thread of the quadrant's two warps passes the same number of
-        // named barriers; after a wait runs out the warps skip the work but keep
-        // the count, so no barrier is left waiting.
-        const int bar_id = 1 + quad;
-        uint32_t g = 0;
+        // The quadrant's three warps pass the same number of named barriers (1..4: new weights);
+        // after a wait runs out they skip the work but keep the count, so no barrier is left
+        // waiting.
+        uint32_t g0 = 0, par = 0;  // tiles before the pass, parity of the unit
         bool dead = false;
-        f32x2 vr[kNB][kHC / 2];  // quadrature weights (times 2^ea) of tracers 0..4 of the B-side kind
-        for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
+        // weights of this thread's cosmology: tracer j, columns 4 c .. 4 c + 3 at vb[j][c][lane]
+        float4 *vb = reinterpret_cast<float4 *>(sV) + bl_;
+        const uint32_t vbs = smem_u32(vb);
+        for (int u = blockIdx.x; u < n_units; u += gridDim.x, par ^= 1) {
             int grp, q0;
             unit_decode(args, u, grp, q0);
             const int a = q0 / args.Rn, rt = (q0 % args.Rn) / kQT;
+            float *sc = s_sc + par * (3 * BLAST_MAX_ELL);
+            // the pair (hi, lo) of tracer j goes to Y[t][es][a][b / 32][group][rt][j][hi, lo][b % 32]:
+            // a warp stores 128 bytes
+            float *yu = args.Y + ((((size_t)a * (args.Bpad / 32) + (b >> 5)) * args.ngr + grp) * args.RT + rt) *
+                                     (size_t)kNB * 64 + lane;
             for (int t = 0; t < args.npass; t++) {  // t: pass (the Y index)
                 const int kindB = pass_kind(t, args.sym);
-                const int offB = kindB ? ng : 0, nB = kindB ? ns : ng;
                 if (t == 0 || kindB != pass_kind(t - 1, args.sym)) {
-                    // weights of the pass's B-side kind (passes of one kind follow each
-                    // other), tracers 5 grp .. 5 grp + 4 of it
-#pragma unroll
-                    for (int j = 0; j < kNB; j++) {
-                        const int jj = kNB * grp + j;
-                        const float4 *src =
-                            (valid && jj < nB)
-                                ? reinterpret_cast<const float4 *>(rq->V32 + (size_t)(offB + jj) * args.Q + q0 + cb)
-                                : nullptr;
-#pragma unroll
-                        for (int c = 0; c < kHC / 4; c++) {
-                            const float4 v = src ? src[c] : make_float4(0.f, 0.f, 0.f, 0.f);
-                            vr[j][2 * c] = pk2(v.x * sa, v.y * sa);
-                            vr[j][2 * c + 1] = pk2(v.z * sa, v.w * sa);
+                    // weights (times 2^ea) of the pass's B-side kind (passes of one kind follow
+                    // each other), tracers 5 grp .. 5 grp + 4 of it, once the quadrant's warps
+                    // have left the old ones: a warp brings every third group of four columns
+                    named_bar_sync(1 + quad, 32 * kEW);
+                    if (t == 0) {
+                        // the unit's tile scales 2^(eG - 16): every quadrant writes the same values; no
+                        // quadrant can be a whole unit ahead of another, so two buffers suffice
+                        for (int i = turn * 32 + lane; i < 3 * args.n_esel; i += 32 * kEW) {
+                            const int tb = i / args.n_esel, es = i - tb * args.n_esel;
+                            sc[tb * BLAST_MAX_ELL + es] =
+                                args.scT[((size_t)tb * args.L + s_esel[es]) * (args.Q / kQT) + q0 / kQT];
                         }
                     }
+                    const ReqDev *rq = b < args.n ? &args.reqs[b] : nullptr;
+                    const int nB = rq ? (kindB ? rq->n_lens : rq->n_clust) - kNB * grp : 0;
+                    const float sa = args.sa[b];
+                    const float *V = rq ? rq->V32 + (size_t)((kindB ? rq->n_clust : 0) + kNB * grp) * args.Q + q0
+                                        : nullptr;
+                    for (int i = turn; i < kNB * (kQT / 4); i += kEW) {
+                        const int j = i / (kQT / 4), c = i % (kQT / 4);
+                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (j < nB) v = *reinterpret_cast<const float4 *>(V + (size_t)j * args.Q + 4 * c);
+                        vb[i * kM] = make_float4(v.x * sa, v.y * sa, v.z * sa, v.w * sa);
+                    }
+                    named_bar_sync(1 + quad, 32 * kEW);
                 }
-                for (int es = 0; es < args.n_esel; es++, g++) {
+                const float *sct = sc + pass_basis(t, args.sym) * BLAST_MAX_ELL;
+                // this warp's tiles of the pass
+                for (int es = (int)((kEW + turn - g0 % kEW) % kEW); es < args.n_esel; es += kEW) {
+                    const uint32_t g = g0 + es;  // tile
                     const int buf = g % kNBUF;
-                    const uint32_t tph = (g / kNBUF) & 1;
-                    // the tile's scale 2^(eG - 16), fetched while the MMA finishes
-                    const float tsc =
-                        (part == 0) ? args.scT[((size_t)pass_basis(t, args.sym) * args.L + s_esel[es]) * (args.Q / kQT) +
-                                               q0 / kQT]
-                                    : 0.f;
                     if (!dead) {
                         bool lost = *abort_flag != 0;
                         // test hook: one warp of CTA 0 waits, with a 20M-cycle limit, on a
                         // barrier nothing completes, so the bounded wait runs out
-                        if (!lost && (int)g == args.trip && blockIdx.x == 0 && warp == 2 &&
+                        if (!lost && (int)g == args.trip && blockIdx.x == 0 && quad == 2 &&
                             !mbar_wait(never, 0, 0, 20000000LL)) {
                             lost = true;
                             atomicExch(args.err, 4);
                             *abort_flag = 1;
                         }
-                        if (!lost && !mbar_wait(&tfull[buf], tph)) {
+                        if (!lost && !mbar_wait(&tfull[g % kFull], (g / kFull) & 1)) {
                             lost = true;
                             atomicExch(args.err, 4);
                             *abort_flag = 1;
                         }
                         dead = __any_sync(0xffffffffu, lost);
                     }
-                    float Sh[NGB], Sl[NGB];
+                    if (dead) continue;
+                    if (!qlive) {  // nothing of this buffer is read
+                        mbar_arrive(&tempty[buf]);
+                        continue;
+                    }
+                    tc_fence_after();
+                    const uint32_t tcol = tmem + lane_addr + buf * (LV * kQT);
+                    // Levels 0..2 are exact multiples of their quanta, so both fast two-sums
+                    // are exact; the small parts add plainly (one rounding)
+                    f32x2 m[kQT / 2], lo[kQT / 2];
 #pragma unroll
-                    for (int j = 0; j < NGB; j++) { Sh[j] = 0.f; Sl[j] = 0.f; }
-                    if (!dead && !qlive) mbar_arrive(&tempty[buf]);  // nothing of this buffer is read
-                    if (!dead && qlive) {
-                        tc_fence_after();
-                        const uint32_t tcol = tmem + lane_addr + buf * (LV * kQT) + cb;
-                        // R-sum of this thread's columns, two columns per packed lane pair, as
-                        // negated unevaluated sums An + Bn: each product V w is split exactly
-                        // (FMA), the two products of a lane pair are added plainly, and each
-                        // addition of those sums keeps its rounding error (two-sum), so the
-                        // sum survives the cancellation of oscillating w
-                        f32x2 An[NGB], Bn[NGB];
+                    for (int s = 0; s < kQT / kCS; s++) {
+                        uint32_t D[LV][kCS];
 #pragma unroll
-                        for (int s = 0; s < kHC / kCS; s++) {
-                            uint32_t D[LV][kCS];
+                        for (int lev = 0; lev < LV; lev++) tmem_ld8(tcol + lev * kQT + s * kCS, D[lev]);
+                        tmem_wait_ld8(D[0]);
 #pragma unroll
-                            for (int lev = 0; lev < LV; lev++) tmem_ld4(tcol + lev * kQT + s * kCS, D[lev]);
-                            tmem_wait_ld4(D[0]);
+                        for (int lev = 1; lev < LV; lev++) reg_fence8(D[lev]);
 #pragma unroll
-                            for (int lev = 1; lev < LV; lev++) reg_fence4(D[lev]);
-                            if (s + 1 == kHC / kCS) {  // every level of this buffer is in registers: release it
-                                tc_fence_before();
-                                mbar_arrive(&tempty[buf]);
+                        for (int h = 0; h < kCS / 2; h++) {
+                            const int x = s * (kCS / 2) + h;
+                            f32x2 d[LV], e1, e2;
+#pragma unroll
+                            for (int lev = 0; lev < LV; lev++)
+                                d[lev] = pk2(__uint_as_float(D[lev][2 * h]), __uint_as_float(D[lev][2 * h + 1]));
+                            fast_two_sum2(d[0], d[1], m[x], e1);
+                            fast_two_sum2(m[x], d[2], m[x], e2);
+                            lo[x] = add2(add2(e1, e2), add2(d[3], d[4]));
+                        }
+                    }
+                    tc_fence_before();  // every level of this buffer is joined: release it
+                    mbar_arrive(&tempty[buf]);
+                    float Sh[kNB], Sl[kNB];
+#pragma unroll
+                    for (int half = 0; half < kQT / kHC; half++) {
+                        // R-sum of the 16 columns, two columns per packed lane pair, as negated
+                        // unevaluated sums An + Bn: each product V w is split exactly (FMA), the two
+                        // products of a lane pair are added plainly, and each addition of those sums
+                        // keeps its rounding error (two-sum), so the sum survives the cancellation of
+                        // oscillating w
+                        f32x2 An[kNB], Bn[kNB];
+                        float4 vn[kNB];  // the next four columns' weights, loaded a step ahead
+#pragma unroll
+                        for (int j = 0; j < kNB; j++) vn[j] = lds4(vbs + (j * (kQT / 4) + half * (kHC / 4)) * (kM * 16));
+#pragma unroll
+                        for (int ch = 0; ch < kHC / 4; ch++) {
+                            const int h0 = half * (kHC / 2) + 2 * ch, h1 = h0 + 1;
+                            const f32x2 mn0 = neg2(m[h0]), mn1 = neg2(m[h1]);
+                            f32x2 v0[kNB], v1[kNB];
+#pragma unroll
+                            for (int j = 0; j < kNB; j++) {
+                                v0[j] = pk2(vn[j].x, vn[j].y);
+                                v1[j] = pk2(vn[j].z, vn[j].w);
                             }
-                            // levels 0..2 are exact multiples of their quanta, so both fast
-                            // two-sums are exact; the small parts add plainly (one rounding)
-                            f32x2 m[kCS / 2], lo[kCS / 2];
+                            if (ch + 1 < kHC / 4) {
 #pragma unroll
-                            for (int h = 0; h < kCS / 2; h++) {
-                                f32x2 d[LV];
-#pragma unroll
-                                for (int lev = 0; lev < LV; lev++)
-                                    d[lev] = pk2(__uint_as_float(D[lev][2 * h]), __uint_as_float(D[lev][2 * h + 1]));
-                                f32x2 e1, e2;
-                                fast_two_sum2(d[0], d[1], m[h], e1);
-                                fast_two_sum2(m[h], d[2], m[h], e2);
-                                const f32x2 small = (LV == 5) ? add2(d[3], d[LV - 1]) : d[3];
-                                lo[h] = add2(add2(e1, e2), small);
+                                for (int j = 0; j < kNB; j++)
+                                    vn[j] = lds4(vbs + (j * (kQT / 4) + half * (kHC / 4) + ch + 1) * (kM * 16));
                             }
 #pragma unroll
-                            for (int ch = 0; ch < kCS / 4; ch++) {
-                                const int h0 = 2 * ch, h1 = 2 * ch + 1;
-                                const f32x2 mn0 = neg2(m[h0]), mn1 = neg2(m[h1]);
-                                const bool first = (s == 0 && ch == 0);
-#pragma unroll
-                                for (int j = 0; j < NGB; j++) {
-                                    const int pc = s * (kCS / 2) + h0;  // packed column pair index
-                                    const f32x2 v0 = vr[j][pc], v1 = vr[j][pc + 1];
-                                    const f32x2 p0 = mul2(v0, mn0), p1 = mul2(v1, mn1);   // -fl(v m)
-                                    const f32x2 e0 = fma2(v0, lo[h0], fma2(v0, m[h0], p0));  // v lo + (v m - fl(v m))
-                                    const f32x2 e1 = fma2(v1, lo[h1], fma2(v1, m[h1], p1));
-                                    const f32x2 ps = add2(p0, p1), pe = add2(e0, e1);
-                                    if (first) {  // the sums start here
-                                        An[j] = ps;
-                                        Bn[j] = neg2(pe);
-                                    } else {
-                                        f32x2 se;
-                                        two_sum2(An[j], ps, An[j], se);
-                                        Bn[j] = add2(Bn[j], sub2(se, pe));
-                                    }
+                            for (int j = 0; j < kNB; j++) {
+                                const f32x2 p0 = mul2(v0[j], mn0), p1 = mul2(v1[j], mn1);   // -fl(v m)
+                                const f32x2 e0 = fma2(v0[j], lo[h0], fma2(v0[j], m[h0], p0));  // v lo + (v m - fl(v m))
+                                const f32x2 e1 = fma2(v1[j], lo[h1], fma2(v1[j], m[h1], p1));
+                                const f32x2 ps = add2(p0, p1), pe = add2(e0, e1);
+                                if (ch == 0) {  // the sums start here
+                                    An[j] = ps;
+                                    Bn[j] = neg2(pe);
+                                } else {
+                                    f32x2 se;
+                                    two_sum2(An[j], ps, An[j], se);
+                                    Bn[j] = add2(Bn[j], sub2(se, pe));
                                 }
                             }
                         }
-                        // both lanes into one pair per tracer: S = -(An.x + An.y) - (Bn.x + Bn.y)
+                        // both lanes into one pair per tracer: S = -(An.x + An.y) - (Bn.x + Bn.y), and
+                        // the halves into one
 #pragma unroll
-                        for (int j = 0; j < NGB; j++) {
+                        for (int j = 0; j < kNB; j++) {
                             const float2 A2 = unpk2(An[j]), B2 = unpk2(Bn[j]);
                             float h, el;
                             two_sum(A2.x, A2.y, h, el);
-                            Sh[j] = -h;
-                            Sl[j] = -__fadd_rn(el, __fadd_rn(B2.x, B2.y));
-                        }
-                    }
-                    // the column parts meet: parts 1.. hand their pairs to part 0 through
-                    // shared memory, double buffered by iteration
-                    float *yq = ybuf + ((size_t)(g & 1) * 4 + quad) * ((kEP - 1) * NGB * 64);
-                    if (part > 0) {
-                        float *yp = yq + (part - 1) * (NGB * 64);
-#pragma unroll
-                        for (int j = 0; j < NGB; j++) { yp[j * 64 + lane] = Sh[j]; yp[j * 64 + 32 + lane] = Sl[j]; }
-                    }
-                    named_bar_sync(bar_id, 32 * kEP);
-                    if (part == 0 && !dead) {
-#pragma unroll
-                        for (int q = 0; q < kEP - 1; q++) {
-                            const float *yp = yq + q * (NGB * 64);
-#pragma unroll
-                            for (int j = 0; j < NGB; j++) {
+                            const float l = -__fadd_rn(el, __fadd_rn(B2.x, B2.y));
+                            if (half == 0) {
+                                Sh[j] = -h;
+                                Sl[j] = l;
+                            } else {
                                 float se;
-                                two_sum(Sh[j], yp[j * 64 + lane], Sh[j], se);
-                                Sl[j] = __fadd_rn(Sl[j], __fadd_rn(se, yp[j * 64 + 32 + lane]));
+                                two_sum(Sh[j], -h, Sh[j], se);
+                                Sl[j] = __fadd_rn(Sl[j], __fadd_rn(se, l));
                             }
                         }
-                        if (valid) {
-                            // times the tile's scale (exact); the pair (hi, lo) of tracer j at
-                            // Y[t][es][a][b / 32][rt][j][hi, lo][b % 32]: a warp stores 128 bytes
-                            float *y = args.Y +
-                                       ((((((size_t)t * args.n_esel + es) * args.X + a) * (args.Bpad / 32) + (b >> 5)) *
-                                             args.ngr + grp) * args.RT + rt) * (size_t)kNB * 64 + lane;
+                    }
+                    if (b < args.n) {
+                        const float tsc = sct[es];  // times the tile's scale (exact)
+                        float *y = yu + ((size_t)t * args.n_esel + es) * args.ystep;
 #pragma unroll
-                            for (int j = 0; j < NGB; j++) { y[j * 64] = Sh[j] * tsc; y[j * 64 + 32] = Sl[j] * tsc; }
-                        }
+                        for (int j = 0; j < kNB; j++) { y[j * 64] = Sh[j] * tsc; y[j * 64 + 32] = Sl[j] * tsc; }
                     }
                 }
+                g0 += args.n_esel;
             }
         }
     }
@@ -1069,6 +1093,7 @@ int launch_contract_tc(blast_plan *p, ReqDev *dreq, int n, const int *d_esel, in
     args.trip = p->test_trip;
     p->test_trip = -1;  // one call only
     args.ngr = (tc_mt(p) + kNB - 1) / kNB;
+    args.ystep = (size_t)args.X * (args.Bpad / 32) * args.ngr * args.RT * kNB * 64;
     if (p->Kst > kKC) {
         // coefficient slice 4 for the shared-memory operand of the p = 4 MMAs
         CUtensorMap mapA4;
