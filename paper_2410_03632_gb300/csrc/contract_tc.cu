@@ -46,10 +46,14 @@
 // eight epilogue warps that held their weights in registers, took half a tile
 // each, met at a barrier and waited for the tile's scale from L2, and one issuer;
 // 1.60 ms so.  150 ragged cosmologies of up to 10+10 tracers (32 ells, 256 x 192
-// nodes, order 96): 6.05 ms and 5.04 ms.
+// nodes, order 96): 6.05 ms and 4.75 ms.
+// A last cosmology tile of at most 64 repeats its cosmologies in the idle lane
+// quadrants, whose warps then take turns with the tiles: one cosmology 0.89 ms
+// without, 0.55 ms with it (and with the passes as units of their own).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <climits>
 #include <cmath>
 #include <cstring>
@@ -67,7 +71,7 @@ constexpr int kNBUF = 2;                  // TMEM accumulator buffers
 constexpr int kEW = 3;                    // epilogue warps per TMEM lane quadrant, tiles in turn
 constexpr int kEpi0 = 4;                  // first epilogue warp (warp 0 TMA, 1 and 2 MMA, 3 spare)
 constexpr int kThreads = 128 + 128 * kEW;
-constexpr int kFull = kNBUF * kEW;        // tile-complete barriers: one per buffer and epilogue warp
+constexpr int kFull = 4 * kEW;            // tile-complete barriers: a multiple of the buffers and of every turn
 constexpr int kHC = kQT / 2;              // columns summed together
 constexpr int kCS = 8;                    // columns per TMEM load step
 constexpr int kNB = 5;                    // tracers per weight group
@@ -75,7 +79,7 @@ constexpr uint32_t kBSliceBytes = kQT * 128;  // 32 rows x 64 bf16
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kCtrlBytes = 256;          // mbarriers, TMEM address, abort flag
 constexpr uint32_t kEselBytes = 4 * BLAST_MAX_ELL;  // selected ells
-constexpr uint32_t kScBytes = 2 * 3 * 4 * BLAST_MAX_ELL;  // tile scales of a unit, two units
+constexpr uint32_t kScBytes = 4 * 3 * 4 * BLAST_MAX_ELL;  // tile scales of a unit, per quadrant
 
 // Compile-time shape of one kernel instance: KC 64-wide K chunks per tile
 // (1: order <= 64, 2: order <= 96), one chunk per stage.
@@ -319,6 +323,8 @@ struct TcArgs {
     const uint16_t *A;   // [S][Bpad][Kst] coefficient slices
     float *Y;            // [npass][n_esel][X][Bpad/32][ngr][RT][5][hi, lo][32] R-tile partial pairs
     size_t ystep;        // floats of Y between ells
+    int cta_full, cta_last;  // CTAs of each full cosmology tile and of the last one
+    int psplit, np_unit;     // parts of the passes (units of a q tile), passes of a unit
     int *err;            // host-mapped error word
     int trip;            // test hook: tile at which CTA 0 waits on a barrier nothing completes (-1 off)
 };
@@ -338,14 +344,34 @@ __host__ __device__ __forceinline__ int pass_kind_a(int pass, int sym)
     return sym ? (pass == 1 || pass == 3) : (pass == 2);
 }
 
-// Work units: (cosmology tile, group of five B-side tracers, 32-column q
-// tile).  A CTA keeps its cosmology tile (the grid is a multiple of nbt), so
-// the coefficient slices stay in TMEM for the whole launch; each unit runs
-// the 3 n_esel (type, ell) tiles of its q tile.
-__device__ __forceinline__ void unit_decode(const TcArgs &a, int u, int &grp, int &q0)
+// Work units of a cosmology tile: (group of five B-side tracers, 32-column q
+// tile, part of the passes).  A CTA keeps its cosmology tile, so the
+// coefficient slices stay in TMEM for the whole launch, and runs the (pass,
+// ell) tiles of every unit it is given.  A last tile with few cosmologies gets
+// fewer CTAs (its tiles are faster).
+struct CtaPlace {
+    int btile, first, step;  // cosmology tile, first unit and the units between
+    __device__ __forceinline__ CtaPlace(const TcArgs &a, int cta)
+    {
+        const int nfull = a.nbt - 1, c = cta - a.cta_full * nfull;
+        if (c < 0) {
+            btile = cta % nfull;
+            first = cta / nfull;
+            step = a.cta_full;
+        } else {
+            btile = nfull;
+            first = c;
+            step = a.cta_last;
+        }
+    }
+};
+
+__device__ __forceinline__ void unit_decode(const TcArgs &a, int u, int &grp, int &q0, int &t0)
 {
-    grp = (u / a.nbt) % a.ngr;
-    q0 = (u / (a.nbt * a.ngr)) * kQT;
+    const int g = u / a.psplit;
+    t0 = (u - g * a.psplit) * a.np_unit;
+    grp = g % a.ngr;
+    q0 = (g / a.ngr) * kQT;
 }
 
 template <int KC>
@@ -368,18 +394,25 @@ k_contract_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ 
     uint32_t *tmem_slot = (uint32_t *)(never + 1);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     int *s_esel = (int *)((unsigned char *)bars + kCtrlBytes);         // selected ells
-    float *s_sc = (float *)((unsigned char *)s_esel + kEselBytes);     // [unit parity][type][ell] tile scales
+    float *s_sc = (float *)((unsigned char *)s_esel + kEselBytes);     // [quadrant][type][ell] tile scales
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int btile = blockIdx.x % args.nbt;
-    const int n_iter_unit = args.npass * args.n_esel;
-    const int n_units = args.nbt * args.ngr * args.nqt;
+    const CtaPlace cta(args, blockIdx.x);
+    const int btile = cta.btile;
+    // Quadrants of 32 TMEM lanes that hold different cosmologies; a tile of at most 64
+    // repeats them in the other quadrants, which then take turns with the tiles: an SM
+    // sub-partition runs one quadrant's epilogue, so without it a small batch leaves three
+    // (two) of four idle while the tile takes as long as a full one.
+    const int live = min(kM, args.n - btile * kM);
+    const int nqb = live <= 32 ? 1 : live <= 64 ? 2 : 4;
+    const int n_iter_unit = args.np_unit * args.n_esel;
+    const int n_units = args.ngr * args.nqt * args.psplit;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; i++) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
         mbar_init(aready, 128);
         for (int i = 0; i < kFull; i++) mbar_init(&tfull[i], 1);
-        for (int i = 0; i < kNBUF; i++) mbar_init(&tempty[i], 128);
+        for (int i = 0; i < kNBUF; i++) mbar_init(&tempty[i], 32 * nqb);
         for (int i = 0; i < kNBUF; i++) mbar_init(&mdone[i], 1);
         mbar_init(a4ready, 1);
         mbar_init(never, 1);
@@ -403,17 +436,20 @@ k_contract_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ 
             if (elect_one()) {
                 mbar_expect_tx(a4ready, C::kA4Bytes);
 #pragma unroll
-                for (int c = 0; c < KC; c++) tma_load_2d(sA4 + c * kM * 128, &mapA4, a4ready, c * kKC, btile * kM);
+                for (int c = 0; c < KC; c++)
+                    for (int q = 0; q < 4; q++)
+                        tma_load_2d(sA4 + (c * kM + q * 32) * 128, &mapA4, a4ready, c * kKC,
+                                    btile * kM + q % nqb * 32);
             }
             __syncwarp();
         }
         uint32_t k = 0;  // stages filled
         bool ok = true;
-        for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-            int grp, q0;
-            unit_decode(args, u, grp, q0);
+        for (int u = cta.first; ok && u < n_units; u += cta.step) {
+            int grp, q0, t0;
+            unit_decode(args, u, grp, q0, t0);
             for (int it = 0; ok && it < n_iter_unit; it++) {
-                const int t = pass_basis(it / args.n_esel, args.sym), e = s_esel[it % args.n_esel];
+                const int t = pass_basis(t0 + it / args.n_esel, args.sym), e = s_esel[it % args.n_esel];
                 const int row = (t * args.L + e) * args.Q + q0;
 #pragma unroll
                 for (int c = 0; c < KC; c++, k++) {
@@ -453,8 +489,8 @@ k_contract_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ 
         const uint32_t acol = args.Kmma / 2;  // TMEM columns per coefficient slice
         const int buf = warp - 1;
         const uint32_t dbase = tm + buf * (LV * kQT);
-        const uint32_t n_tiles = blockIdx.x < n_units ? (n_units - 1 - blockIdx.x) / gridDim.x * n_iter_unit + n_iter_unit
-                                                      : 0;
+        const uint32_t n_tiles =
+            cta.first < n_units ? (uint32_t)((n_units - 1 - cta.first) / cta.step + 1) * n_iter_unit : 0;
         int st = buf * KC;  // stage and its lap's parity
         uint32_t ph = 0;
         for (uint32_t g = buf; ok && g < n_tiles; g += kNBUF) {
@@ -518,10 +554,10 @@ k_contract_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ 
         const int quad = warp & 3;   // lanes 32 quad .. 32 quad + 31 are readable by this warp
         const int turn = (warp - kEpi0) >> 2;
         const int bl_ = quad * 32 + lane;
-        const int b = btile * kM + bl_;
-        // a quadrant whose 32 lanes are all padding (a batch smaller than the
-        // tile) only keeps the buffer hand-off in step
-        const bool qlive = btile * kM + quad * 32 < args.n;
+        const int b = btile * kM + quad % nqb * 32 + lane;  // cosmology
+        const uint32_t nrep = 4 / nqb, rix = quad / nqb;     // tiles of this quadrant: g % nrep == rix
+        // a quadrant whose 32 lanes are all padding only keeps the buffer hand-off in step
+        const bool qlive = btile * kM + quad % nqb * 32 < args.n;
         const uint32_t lane_addr = ((uint32_t)(quad * 32)) << 16;
         if (turn == 0) {
             // coefficient slices of cosmology b -> TMEM lane b, columns kACol + (Kmma/2) p ..
@@ -543,30 +579,28 @@ k_contract_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ 
         // The quadrant's three warps pass the same number of named barriers (1..4: new weights);
         // after a wait runs out they skip the work but keep the count, so no barrier is left
         // waiting.
-        uint32_t g0 = 0, par = 0;  // tiles before the pass, parity of the unit
+        uint32_t g0 = 0;  // tiles before the pass
         bool dead = false;
         // weights of this thread's cosmology: tracer j, columns 4 c .. 4 c + 3 at vb[j][c][lane]
         float4 *vb = reinterpret_cast<float4 *>(sV) + bl_;
         const uint32_t vbs = smem_u32(vb);
-        for (int u = blockIdx.x; u < n_units; u += gridDim.x, par ^= 1) {
-            int grp, q0;
-            unit_decode(args, u, grp, q0);
+        float *sc = s_sc + quad * (3 * BLAST_MAX_ELL);
+        for (int u = cta.first; u < n_units; u += cta.step) {
+            int grp, q0, t0;
+            unit_decode(args, u, grp, q0, t0);
             const int a = q0 / args.Rn, rt = (q0 % args.Rn) / kQT;
-            float *sc = s_sc + par * (3 * BLAST_MAX_ELL);
             // the pair (hi, lo) of tracer j goes to Y[t][es][a][b / 32][group][rt][j][hi, lo][b % 32]:
             // a warp stores 128 bytes
             float *yu = args.Y + ((((size_t)a * (args.Bpad / 32) + (b >> 5)) * args.ngr + grp) * args.RT + rt) *
                                      (size_t)kNB * 64 + lane;
-            for (int t = 0; t < args.npass; t++) {  // t: pass (the Y index)
+            for (int t = t0; t < t0 + args.np_unit; t++) {  // t: pass (the Y index)
                 const int kindB = pass_kind(t, args.sym);
-                if (t == 0 || kindB != pass_kind(t - 1, args.sym)) {
+                if (t == t0 || kindB != pass_kind(t - 1, args.sym)) {
                     // weights (times 2^ea) of the pass's B-side kind (passes of one kind follow
                     // each other), tracers 5 grp .. 5 grp + 4 of it, once the quadrant's warps
                     // have left the old ones: a warp brings every third group of four columns
                     named_bar_sync(1 + quad, 32 * kEW);
-                    if (t == 0) {
-                        // the unit's tile scales 2^(eG - 16): every quadrant writes the same values; no
-                        // quadrant can be a whole unit ahead of another, so two buffers suffice
+                    if (t == t0) {  // the unit's tile scales 2^(eG - 16), a copy for each quadrant
                         for (int i = turn * 32 + lane; i < 3 * args.n_esel; i += 32 * kEW) {
                             const int tb = i / args.n_esel, es = i - tb * args.n_esel;
                             sc[tb * BLAST_MAX_ELL + es] =
@@ -588,14 +622,15 @@ k_contract_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ 
                 }
                 const float *sct = sc + pass_basis(t, args.sym) * BLAST_MAX_ELL;
                 // this warp's tiles of the pass
-                for (int es = (int)((kEW + turn - g0 % kEW) % kEW); es < args.n_esel; es += kEW) {
+                const uint32_t step = nrep * kEW, mine = rix + nrep * turn;
+                for (int es = (int)((step + mine - g0 % step) % step); es < args.n_esel; es += step) {
                     const uint32_t g = g0 + es;  // tile
                     const int buf = g % kNBUF;
                     if (!dead) {
                         bool lost = *abort_flag != 0;
                         // test hook: one warp of CTA 0 waits, with a 20M-cycle limit, on a
                         // barrier nothing completes, so the bounded wait runs out
-                        if (!lost && (int)g == args.trip && blockIdx.x == 0 && quad == 2 &&
+                        if (!lost && (int)g == args.trip && blockIdx.x == 0 && quad % nqb == 0 &&
                             !mbar_wait(never, 0, 0, 20000000LL)) {
                             lost = true;
                             atomicExch(args.err, 4);
@@ -987,17 +1022,31 @@ int tc_npass(const blast_plan *p) { return p->r_form == 1 ? 4 : 3; }
 size_t tc_u_bytes(const blast_plan *p, int Bpad) { return (size_t)Bpad * p->X * 4 * tc_mt(p) * 4; }
 
 template <int KC>
-int launch_contract_inst(blast_plan *p, const CUtensorMap &mapB, const CUtensorMap &mapA4, const TcArgs &args,
+int launch_contract_inst(blast_plan *p, const CUtensorMap &mapB, const CUtensorMap &mapA4, TcArgs args,
                          cudaStream_t s)
 {
     using C = TcCfg<KC>;
-    const int sms = p->sms;
-    const int units = args.nbt * args.ngr * args.nqt;
-    // persistent CTAs: the autotuned count when set, else every SM
-    int grid = p->tune.grid > 0 ? p->tune.grid : sms / args.nbt * args.nbt;
-    grid = grid / args.nbt * args.nbt;
-    if (grid > units) grid = units;
+    // persistent CTAs: the autotuned count when set, else every SM.  A last cosmology
+    // tile of at most 32 (64) takes less than a full one, measured 1630 (1810) cycles of
+    // 2470 a basis tile at order 64 and 2250 of 2650 at order 96, where the MMAs bound it
+    const int units = args.ngr * args.nqt, nfull = args.nbt - 1, last = args.n - nfull * kM;
+    const double share = last > 64 ? 1.0 : KC == 2 ? 0.85 : last <= 32 ? 0.66 : 0.73;
+    int grid = p->tune.grid > 0 ? p->tune.grid : p->sms;
     if (grid < args.nbt) grid = args.nbt;
+    args.cta_full = (int)(grid / (nfull + share));
+    args.cta_last = grid - args.cta_full * nfull;
+    if (args.cta_last < 1) { args.cta_full--; args.cta_last += nfull; }
+    // a q tile's passes as units of their own where that fills the last round of CTAs
+    // better (by 3 % or more: each unit loads its weights)
+    auto rounds = [&](int parts) {
+        auto up = [&](int ctas) { return (units * parts + ctas - 1) / ctas; };
+        return std::max(nfull ? up(args.cta_full) : 0, (int)std::ceil(up(args.cta_last) * (nfull ? share : 1.0)));
+    };
+    args.psplit = rounds(args.npass) < 0.97 * args.npass * rounds(1) ? args.npass : 1;
+    args.np_unit = args.npass / args.psplit;
+    if (args.cta_full > units * args.psplit) args.cta_full = units * args.psplit;
+    if (args.cta_last > units * args.psplit) args.cta_last = units * args.psplit;
+    grid = args.cta_full * nfull + args.cta_last;
     k_contract_tc<KC><<<grid, kThreads, C::kSmem, s>>>(mapB, mapA4, args);
     BL_CUDA(cudaGetLastError());
     return BLAST_OK;
@@ -1097,7 +1146,7 @@ int launch_contract_tc(blast_plan *p, ReqDev *dreq, int n, const int *d_esel, in
     if (p->Kst > kKC) {
         // coefficient slice 4 for the shared-memory operand of the p = 4 MMAs
         CUtensorMap mapA4;
-        if ((rc = make_map2d(&mapA4, A + (size_t)(kS - 1) * Bpad * p->Kst, p->Kst, Bpad, kM))) return rc;
+        if ((rc = make_map2d(&mapA4, A + (size_t)(kS - 1) * Bpad * p->Kst, p->Kst, Bpad, 32))) return rc;
         return launch_contract_inst<2>(p, mapB, mapA4, args, s);
     }
     return launch_contract_inst<1>(p, mapB, mapB, args, s);
