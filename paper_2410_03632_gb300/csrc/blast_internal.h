@@ -11,6 +11,7 @@
 
 #define BLAST_MAX_ELL 128
 #define BLAST_MAX_TRACERS 32
+#define BLAST_MAX_NR 512     // n_R of a plan
 #define BLAST_TC_SLICES 5   // 8-bit fixed-point slices per operand on the tensor-core path
 
 // Status helpers -------------------------------------------------------------

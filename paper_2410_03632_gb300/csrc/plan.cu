@@ -191,7 +191,7 @@ extern "C" int blast_plan_create(const blast_plan_desc *d, blast_plan **out)
     }
     if (d->n_chi < 4 || !(d->chi_min > 0) || !(d->chi_max > d->chi_min)) return BLAST_EINVAL;
     if (d->r_form != 0 && d->r_form != 1) return BLAST_EINVAL;
-    if (d->n_R < 2 || d->n_R % 2 || d->n_R > 512) return BLAST_EINVAL;
+    if (d->n_R < 2 || d->n_R % 2 || d->n_R > BLAST_MAX_NR) return BLAST_EINVAL;
     if (d->r_form == 0 && (!(d->R_min > 0) || !(d->R_min < 1.0) || !(d->R_max > 1.0))) return BLAST_EINVAL;
     if (d->n_cheb < 2 || d->n_cheb > 128 || !(d->k_min > 0) || !(d->k_max > d->k_min)) return BLAST_EINVAL;
     if (d->k_map < 0 || d->k_map > 1) return BLAST_EINVAL;
