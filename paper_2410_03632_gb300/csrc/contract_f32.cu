@@ -2,28 +2,31 @@
 //
 //   w_b(q) = sum_n a_b[n] T~[t][l][n][q],  Y_b(t, l, a, j) = sum_r V_bj(a, r) w_b(a n_R + r).
 //
-// A block of two warps owns one chi node of one (type, ell) and BB
-// cosmologies.  A thread keeps w of NQ R nodes for all of them, so a basis
+// A block of two warps owns one chi node, eight (type, ell) pairs in turn and
+// BB cosmologies.  A thread keeps w of NQ R nodes for all of them, so a basis
 // value is loaded once per BB multiply-adds and a coefficient (a broadcast from
 // shared memory) once per NQ, and the sums over lanes are halved in width at
-// every step: BB values cost BB shuffles, not 5 BB.  Blocks run over the
-// cosmology groups first (they share the basis tile in L2), then over (type,
-// ell) (they share the weights), then over chi nodes.
+// every step: BB values cost BB shuffles, not 5 BB.  Two cosmologies share a
+// packed multiply-add.  Blocks run over the cosmology groups first (they share
+// the basis tile in L2), then over (type, ell) (they share the weights), then
+// over chi nodes.
 //
 // Order of the sums: n ascending, then the R nodes of a lane (r = lane + 32 v +
 // 128 k, v = 0..3) in ascending k, the lanes of each v in the tree 16, 8, 4, 2,
 // 1, and v = 0..3 in turn.  It depends on nothing but n_R, so a cosmology's
 // bits are the same in every batch and for every BB and NQ.
 //
-// Bound by issue: multiply-adds, and the loads and shuffles between them.  48
-// cosmologies (64 ells, 128 x 128 nodes, order 64, 5+5 tracers) take 1.2 ms;
+// Bound by issue and L2 latency (128 registers leave 16 warps an SM).  48
+// cosmologies (64 ells, 128 x 128 nodes, order 64, 5+5 tracers) take 1.07 ms;
 // one block per cosmology and node, which re-read the basis from L2 for each
-// and shuffled five times per tracer, took 19 ms.
+// and shuffled five times per tracer, took 19 ms; without the packed pairs and
+// the shared coefficients it was 1.22 ms.
 #include "blast_internal.h"
 
 namespace {
 
 constexpr int kThreads = 64;
+constexpr int kSpan = 8;   // (type, ell) pairs of a block, which share its coefficients
 
 // Sum over the 32 lanes of each of the BB values x[0..BB): the width halves
 // while more than one value is left.  Returns the sum of value `mine`.
@@ -47,6 +50,23 @@ __device__ __forceinline__ float lane_sums(float (&x)[BB], int lane, int &mine)
     return x[0];
 }
 
+// Two cosmologies in one 64-bit register pair: one instruction multiplies and
+// adds for both, each rounded as alone.
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pair(float x, float y)
+{
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+    return d;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
 template <int BB, int NQ>
 __global__ void __launch_bounds__(kThreads)
 k_contract_f32(const ReqDev *__restrict__ reqs, int n, const float *__restrict__ basis, int L, int N, int X, int Rn,
@@ -54,90 +74,113 @@ k_contract_f32(const ReqDev *__restrict__ reqs, int n, const float *__restrict__
 {
     extern __shared__ float4 sm4[];
     float *as = reinterpret_cast<float *>(sm4);  // [N][BB]
-    float *red = as + (size_t)N * BB;            // [tracer][v][BB]
-    __shared__ const float *sV[BB];
-    __shared__ int sB[BB];
-    const int g = blockIdx.x % ngr, rest = blockIdx.x / ngr;
-    const int a = rest / (3 * n_esel), tl = rest - a * 3 * n_esel;
-    const int t = tl / n_esel, es = tl - t * n_esel, e = esel[es];
+    float *red = as + (size_t)N * BB;            // [parity][tracer][v][BB]
+    constexpr int PB = (BB + 1) / 2;             // pairs of cosmologies (one of a single one is empty)
+    __shared__ __align__(16) int sV[3][2 * PB];  // a cosmology's list of a type, in floats from the first one's weights
+    __shared__ int sB[3][BB], sE[kSpan];
+    __shared__ const float *sA[BB];
+    const int g = blockIdx.x % ngr, rest = blockIdx.x / ngr, ntl = 3 * n_esel;
+    const int nspan = (ntl + kSpan - 1) / kSpan, a = rest / nspan, tl0 = (rest - a * nspan) * kSpan;
     const int b0 = g * BB, nb = min(BB, n - b0), Q = X * Rn;
     const int tid = threadIdx.x, lane = tid & 31, pw = tid >> 5;
-    const bool both = sym && t == 1;
-    for (int i = tid; i < N * BB; i += kThreads) {
-        const int b = i % BB;
-        as[i] = b < nb ? reqs[b0 + b].a32[i / BB] : 0.f;
-    }
-    if (tid < BB) {
+    const float *V0 = reqs[b0].V32 + (size_t)a * Rn;
+    if (tid < 2 * PB) {
         const bool live = tid < nb;
-        const int ng = live ? reqs[b0 + tid].n_clust : 0, ns = live ? reqs[b0 + tid].n_lens : 0;
-        sB[tid] = t == 0 ? ng : both ? ng + ns : ns;
-        sV[tid] = live ? reqs[b0 + tid].V32 + (size_t)(t == 0 || both ? 0 : ng) * Q + (size_t)a * Rn : nullptr;
+        const ReqDev &rq = reqs[b0 + (live ? tid : 0)];
+        const int ng = rq.n_clust, ns = rq.n_lens, off = (int)(rq.V32 + (size_t)a * Rn - V0);
+        if (tid < BB) sA[tid] = rq.a32;
+        for (int t = 0; t < 3; t++) {
+            const bool both = sym && t == 1;
+            sV[t][tid] = off + (t == 0 || both ? 0 : ng * Q);
+            if (tid < BB) sB[t][tid] = !live ? 0 : t == 0 ? ng : both ? ng + ns : ns;
+        }
+    }
+    if (tid < kSpan && tl0 + tid < ntl) sE[tid] = esel[(tl0 + tid) % n_esel];
+    __syncthreads();
+    for (int i = tid; i < N * BB; i += kThreads) {
+        const int b = i / N, k = i - b * N;
+        as[k * BB + b] = b < nb ? __ldg(sA[b] + k) : 0.f;
     }
     __syncthreads();
-    int most = 0;
-#pragma unroll
-    for (int b = 0; b < BB; b++) most = max(most, sB[b]);
-
-    float w[BB][NQ];
-#pragma unroll
-    for (int b = 0; b < BB; b++)
-#pragma unroll
-        for (int i = 0; i < NQ; i++) w[b][i] = 0.f;
-    const float *Tb = basis + ((size_t)t * L + e) * N * Q + (size_t)a * Rn;
     int at[NQ];  // past the end: the last node again, not used
 #pragma unroll
     for (int i = 0; i < NQ; i++) at[i] = min(32 * (pw + 2 * i) + lane, Rn - 1);
+    for (int x = 0; x < kSpan && tl0 + x < ntl; x++) {
+        const int tl = tl0 + x, t = tl / n_esel, es = tl - t * n_esel, e = sE[x];
+        float *redx = red + (x & 1) * (MT * 4 * BB);
+        int most = 0;
+#pragma unroll
+        for (int b = 0; b < BB; b++) most = max(most, sB[t][b]);
+        f32x2 w[PB][NQ];
+#pragma unroll
+        for (int b = 0; b < PB; b++)
+#pragma unroll
+            for (int i = 0; i < NQ; i++) w[b][i] = 0;
+        const float *Tb = basis + ((size_t)t * L + e) * N * Q + (size_t)a * Rn;
 #pragma unroll 4
-    for (int k = 0; k < N; k++) {
-        float tv[NQ], av[BB];
+        for (int k = 0; k < N; k++) {
+            f32x2 tv[NQ], av[PB];
 #pragma unroll
-        for (int i = 0; i < NQ; i++) tv[i] = __ldg(Tb + (size_t)k * Q + at[i]);
-        if constexpr (BB % 4 == 0) {
-#pragma unroll
-            for (int b = 0; b < BB; b += 4) {
-                const float4 v = *reinterpret_cast<const float4 *>(as + (size_t)k * BB + b);
-                av[b] = v.x; av[b + 1] = v.y; av[b + 2] = v.z; av[b + 3] = v.w;
+            for (int i = 0; i < NQ; i++) {
+                const float x = __ldg(Tb + (size_t)k * Q + at[i]);
+                tv[i] = pair(x, x);
             }
-        } else {
+            if constexpr (BB % 4 == 0) {
 #pragma unroll
-            for (int b = 0; b < BB; b++) av[b] = as[(size_t)k * BB + b];
-        }
-#pragma unroll
-        for (int b = 0; b < BB; b++)
-#pragma unroll
-            for (int i = 0; i < NQ; i++) w[b][i] = fmaf(av[b], tv[i], w[b][i]);
-    }
-    for (int j = 0; j < most; j++) {
-        float v[BB][NQ];
-#pragma unroll
-        for (int b = 0; b < BB; b++)
-#pragma unroll
-            for (int i = 0; i < NQ; i++) v[b][i] = j < sB[b] ? __ldg(sV[b] + (size_t)j * Q + at[i]) : 0.f;
-#pragma unroll
-        for (int p = 0; p < 2 && p < NQ; p++) {
-            const int vw = pw + 2 * p;
-            if (32 * vw >= Rn) break;
-            float part[BB];
-#pragma unroll
-            for (int b = 0; b < BB; b++) {
-                part[b] = 0.f;
-#pragma unroll
-                for (int i = p; i < NQ; i += 2)
-                    if (32 * (pw + 2 * i) + lane < Rn) part[b] = fmaf(v[b][i], w[b][i], part[b]);
+                for (int b = 0; b < PB; b += 2) {
+                    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(as + (size_t)k * BB + 2 * b);
+                    av[b] = v.x;
+                    av[b + 1] = v.y;
+                }
+            } else {
+                av[0] = pair(as[k], 0.f);
             }
-            int mine;
-            const float s = lane_sums<BB>(part, lane, mine);
-            if (lane % (32 / BB) == 0) red[(j * 4 + vw) * BB + mine] = s;
+#pragma unroll
+            for (int b = 0; b < PB; b++)
+#pragma unroll
+                for (int i = 0; i < NQ; i++) w[b][i] = fma2(av[b], tv[i], w[b][i]);
         }
-    }
-    __syncthreads();
-    const int nv = min(4, (Rn + 31) / 32);
-    for (int i = tid; i < most * BB; i += kThreads) {
-        const int j = i / BB, b = i % BB;
-        if (j >= sB[b]) continue;
-        float s = 0.f;
-        for (int v = 0; v < nv; v++) s += red[(j * 4 + v) * BB + b];
-        Y[((((size_t)(b0 + b) * 3 + t) * n_esel + es) * X + a) * MT + j] = s;
+        // Rows past a cosmology's own tracers lie in its work space (sized for the plan's
+        // counts); what comes of them is not written.
+        for (int j = 0; j < most; j++) {
+            f32x2 v[PB][NQ];
+            const float *Vj = V0 + (size_t)j * Q;
+#pragma unroll
+            for (int b = 0; b < PB; b++) {
+                const int2 off = *reinterpret_cast<const int2 *>(&sV[t][2 * b]);
+#pragma unroll
+                for (int i = 0; i < NQ; i++)
+                    v[b][i] = pair(__ldg(Vj + (off.x + at[i])), BB > 1 ? __ldg(Vj + (off.y + at[i])) : 0.f);
+            }
+#pragma unroll
+            for (int p = 0; p < 2 && p < NQ; p++) {
+                const int vw = pw + 2 * p;
+                if (32 * vw >= Rn) break;
+                f32x2 part[PB];
+#pragma unroll
+                for (int b = 0; b < PB; b++) {
+                    part[b] = 0;
+#pragma unroll
+                    for (int i = p; i < NQ; i += 2)
+                        if (32 * (pw + 2 * i) + lane < Rn) part[b] = fma2(v[b][i], w[b][i], part[b]);
+                }
+                float x[BB];
+#pragma unroll
+                for (int b = 0; b < BB; b++) x[b] = __uint_as_float((uint32_t)(part[b / 2] >> (32 * (b & 1))));
+                int mine;
+                const float s = lane_sums<BB>(x, lane, mine);
+                if (lane % (32 / BB) == 0) redx[(j * 4 + vw) * BB + mine] = s;
+            }
+        }
+        __syncthreads();
+        const int nv = min(4, (Rn + 31) / 32);
+        for (int i = tid; i < most * BB; i += kThreads) {
+            const int j = i / BB, b = i % BB;
+            if (j >= sB[t][b]) continue;
+            float s = 0.f;
+            for (int v = 0; v < nv; v++) s += redx[(j * 4 + v) * BB + b];
+            Y[((((size_t)(b0 + b) * 3 + t) * n_esel + es) * X + a) * MT + j] = s;
+        }
     }
 }
 
@@ -145,8 +188,9 @@ template <int BB, int NQ>
 int launch(blast_plan *p, const ReqDev *dreq, int n, const int *d_esel, int n_esel, float *Y, cudaStream_t s)
 {
     const int ngr = (n + BB - 1) / BB;
-    const size_t smem = sizeof(float) * ((size_t)p->N * BB + (size_t)p->max_tr * 4 * BB);  // at most 16 KB
-    k_contract_f32<BB, NQ><<<(unsigned)ngr * p->X * 3 * n_esel, kThreads, smem, s>>>(
+    const size_t smem = sizeof(float) * ((size_t)p->N * BB + (size_t)p->max_tr * 8 * BB);  // at most 24 KB
+    const int nspan = (3 * n_esel + kSpan - 1) / kSpan;
+    k_contract_f32<BB, NQ><<<(unsigned)ngr * p->X * nspan, kThreads, smem, s>>>(
         dreq, n, p->T32, p->L, p->N, p->X, p->Rn, d_esel, n_esel, p->max_tr, p->r_form == 1, ngr, Y);
     BL_CUDA(cudaGetLastError());
     return BLAST_OK;
