@@ -5,16 +5,60 @@
 //   T~[t n][l, q] = sum_m A[m][t n] B_l[m][q],  A = w_m f_t(k_m) T_n(x_m),
 //   B_l[m][q]    = j_l(k_m chi_a) j_l(k_m R_r chi_a),
 // with B generated on chip from spherical Bessel recurrences in FP64.
+//
+// The GEMM runs as exact integer products on the FP16 tensor cores (eight 8-bit
+// digits an operand, eight exact levels; contract_fx.cu states the arithmetic),
+// over windows of 56 k nodes: in a window every row of A and every column of B
+// has its own exponent, the window's sum is exact in the levels up to the
+// dropped ones (2^-59 of its largest product), and windows add in FP64.  What is
+// left on the FP64 pipe (two multiply-adds a clock and SM) are the recurrences,
+// a product per entry of B and an addition per output and window.
+//
+// Bound by the recurrences.  16 ells to 200, 38 x 64 nodes, order 32, 65,537 k
+// nodes: 0.31 s (with the GEMM in FP64 multiply-adds and 2l + 1 counted up in
+// FP64 0.81 s); error against an independent FP64 evaluation 2e-15 (9e-15).
 #include <cmath>
 
 #include "blast_internal.h"
+#include "fx.h"
+#include "tc_ptx.h"
 
 namespace {
 
 constexpr int kG = 8;     // plan ells per CTA (one group)
 constexpr int kRT = 8;    // R nodes per CTA
-constexpr int kMC = 28;   // k nodes per chunk: (1 + kRT) * kMC = 252 Bessel chains per chunk
-constexpr int kThreads = 256;
+constexpr int kMC = 56;   // k nodes per window: (1 + kRT) * kMC = 504 Bessel chains
+constexpr int kKS = kMC / 8;              // MMA K steps of a window (8 k nodes, two digits each)
+constexpr int kWork = 512;                // worker threads; then the A loader and the MMA issuer
+constexpr int kThreads = kWork + 64;
+constexpr int kCols = kG * kRT;           // columns of a CTA, in groups of 16
+constexpr int kRows = 16 * kLev;          // rows of a column group's operand, TMEM columns of its levels
+constexpr uint32_t kGroupBytes = (kMC / 4) * kRows * 16;  // a column group's digits: [k-group of 4][row][16 B]
+constexpr uint32_t kAStep = 4 * 2 * 128 * 16;  // A's digits of a K step: [pair][k-group][128 rows][16 B]
+constexpr int kARing = 3;
+
+struct BasisCtl {
+    uint64_t afull[kARing], aempty[kARing], bready, dfull, dempty, mdone;
+    uint32_t tmem;
+    int abort;
+    int colmax[2][kCols];  // biased exponent of a column's largest entry, by parity of the window
+    int lg[kG];
+    double lgr[kG];
+};
+constexpr size_t kBasisSmem = 1024 + (kCols / 16) * kGroupBytes + kARing * kAStep +
+                              sizeof(double) * (1 + kRT) * kMC * kG + sizeof(BasisCtl);
+
+// k as FP64, 0 < k < 2^31, without the FP64 pipe (a conversion costs a
+// recurrence step as much as its multiply-add).
+__device__ __forceinline__ double fp64_of(int k)
+{
+    const int z = __clz(k);
+    const uint32_t m = (uint32_t)k << z;
+    return __hiloint2double((int)(((uint32_t)(1054 - z) << 20) | ((m >> 11) & 0xfffffu)), (int)(m << 21));
+}
+
+// |f| > 1e200 (up to the low 32 bits of the limit), without the FP64 pipe.
+__device__ __forceinline__ bool is_huge(double f) { return (__double2hiint(f) & 0x7fffffff) > 0x6974e718; }
 
 // A[m][t*N + n] = w_m f_t(k_m) T_n(x(k_m)); T_n by the three-term recurrence.
 __global__ void k_basis_A(const double *__restrict__ kq, const double *__restrict__ wq, int Nk, int N,
@@ -62,10 +106,8 @@ __device__ void jl_group(double x, const int *lg, int ng, double *out)
         double jm = j0, jc = j1;
         int gi = 0;
         while (gi < ng && lg[gi] <= 1) { out[gi] = (lg[gi] == 0) ? j0 : j1; gi++; }
-        double dl = 3.0;  // 2l + 1 at l = 1, exact in double
         for (int l = 1; l < lhi; l++) {
-            double jn = (dl * inv) * jc - jm;  // j_{l+1}
-            dl += 2.0;
+            double jn = (fp64_of(2 * l + 1) * inv) * jc - jm;  // j_{l+1}
             jm = jc;
             jc = jn;
             if (gi < ng && l + 1 == lg[gi]) { out[gi] = jc; gi++; }
@@ -75,14 +117,12 @@ __device__ void jl_group(double x, const int *lg, int ng, double *out)
     const int l0 = lhi + 20 + (int)(10.0 * cbrt((double)lhi));
     double fp = 0.0, f = 1e-200;
     int gi = ng - 1;
-    double dl = 2.0 * l0 + 1.0;  // exact in double
     for (int l = l0; l > 0; l--) {
         if (gi >= 0 && l == lg[gi]) { out[gi] = f; gi--; }
-        double fm = (dl * inv) * f - fp;  // f_{l-1}
-        dl -= 2.0;
+        double fm = (fp64_of(2 * l + 1) * inv) * f - fp;  // f_{l-1}
         fp = f;
         f = fm;
-        if ((l & 3) == 0 && fabs(f) > 1e200) {
+        if ((l & 3) == 0 && is_huge(f)) {
             f *= 1e-200;
             fp *= 1e-200;
 #pragma unroll
@@ -216,92 +256,273 @@ __device__ double jnu_real(double nu, double x)
     return rec * (j0 * f + j1 * fp) / ((f * f + fp * fp) * mx);
 }
 
-template <int ROWS>
-__global__ void __launch_bounds__(kThreads)
-k_basis_gemm(const double *__restrict__ A, const double *__restrict__ kq, int Nk, int N,
-             const double *__restrict__ ell, int real_ell, int L, int e0, const double *__restrict__ chi,
-             const double *__restrict__ R, int Rn, int Q, double *__restrict__ T)
+// Digits of A: rows t N + n of 128-row tiles, window by window, each row with
+// its own exponent in a window; the layout is the MMA operand's, one 16 KB block
+// per (row tile, window, K step).
+__global__ void __launch_bounds__(128)
+k_basis_A_digits(const double *__restrict__ A, int Nk, int rows3, int nwin, uint4 *__restrict__ dig,
+                 uint16_t *__restrict__ ea)
 {
-    extern __shared__ double sm[];
-    const int rows3 = 3 * N;
-    double *As = sm;                           // [kMC][3N]
-    double *Jv = As + kMC * rows3;             // [(1+kRT) kMC][kG]
-    double *Bp = Jv + (1 + kRT) * kMC * kG;    // [kMC][kG*kRT]
-    __shared__ int lg[kG];
-    __shared__ double lgr[kG];
+    const int win = blockIdx.x, mt = blockIdx.y, row = mt * 128 + threadIdx.x, m0 = win * kMC;
+    const bool live = row < rows3;
+    int mx = 0;
+    for (int i = 0; i < kMC; i++)
+        if (live && m0 + i < Nk) mx = max(mx, (__double2hiint(A[(size_t)(m0 + i) * rows3 + row]) >> 20) & 0x7ff);
+    const int M = mx < 70 ? kNone : mx;
+    ea[((size_t)mt * nwin + win) * 128 + threadIdx.x] = (uint16_t)M;
+    const uint32_t top = fx_top(M);
+    uint4 *dst = dig + ((size_t)mt * nwin + win) * kKS * (kAStep / 16) + threadIdx.x;
+    for (int kg = 0; kg < kMC / 4; kg++) {
+        uint32_t w[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const int m = m0 + kg * 4 + i;
+            fx_pairs<false>(live && m < Nk ? A[(size_t)m * rows3 + row] : 0.0, top, w[0][i], w[1][i], w[2][i], w[3][i]);
+        }
+#pragma unroll
+        for (int p = 0; p < 4; p++)
+            dst[(size_t)(kg >> 1) * (kAStep / 16) + (p * 2 + (kg & 1)) * 128] =
+                make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
+    }
+}
 
-    const int tid = threadIdx.x;
-    const int a = blockIdx.y;
-    const int r0 = blockIdx.x * kRT;
-    const int ng = min(kG, L - e0);
+// MMA with both operands in shared memory.
+__device__ __forceinline__ void umma_f16_ss(uint32_t d_tmem, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
+        ::"r"(d_tmem), "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+}
+
+// A CTA owns eight R nodes of a chi node and a group of eight ells: 64 columns,
+// 128-row tiles of A in turn.  Per window the workers run the recurrences, then
+// take the previous window's sums out of TMEM, then write the digits of the
+// products j j for the MMAs, which run beside the next window's recurrences.
+__global__ void __launch_bounds__(kThreads, 1)
+k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int Mt, int nwin,
+           const double *__restrict__ kq, int Nk, int N, const double *__restrict__ ell, int real_ell, int L,
+           const double *__restrict__ chi, const double *__restrict__ R, int Rn, int Q, double *__restrict__ T, int *err)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *sB = (unsigned char *)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);  // [group][k-group][row][16 B]
+    unsigned char *sA = sB + (kCols / 16) * kGroupBytes;                                  // [ring][K step block]
+    double *Jv = reinterpret_cast<double *>(sA + kARing * kAStep);                        // [(1 + kRT) kMC][kG]
+    BasisCtl *ctl = reinterpret_cast<BasisCtl *>(Jv + (1 + kRT) * kMC * kG);
+    volatile int *abort_flag = &ctl->abort;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int r0 = blockIdx.x * kRT, a = blockIdx.y, e0 = blockIdx.z * kG, ng = min(kG, L - e0);
+
+    if (tid == 0) {
+        for (int i = 0; i < kARing; i++) { mbar_init(&ctl->afull[i], 1); mbar_init(&ctl->aempty[i], 1); }
+        mbar_init(&ctl->bready, kWork);
+        mbar_init(&ctl->dfull, 1);
+        mbar_init(&ctl->dempty, kWork);
+        mbar_init(&ctl->mdone, 1);
+        ctl->abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     if (tid < kG) {
-        lgr[tid] = (tid < ng) ? ell[e0 + tid] : 0.0;
-        lg[tid] = (int)lgr[tid];
+        ctl->lgr[tid] = (tid < ng) ? ell[e0 + tid] : 0.0;
+        ctl->lg[tid] = (int)ctl->lgr[tid];
     }
-    const double chia = chi[a];
-    const int rb = tid >> 3, cb = tid & 7;
-    double acc[ROWS][kG];
-#pragma unroll
-    for (int i = 0; i < ROWS; i++)
-#pragma unroll
-        for (int g = 0; g < kG; g++) acc[i][g] = 0.0;
+    if (warp == kWork / 32 + 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem)),
+                     "r"(512u));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    tc_fence_before();
     __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = ctl->tmem;
 
-    for (int m0 = 0; m0 < Nk; m0 += kMC) {
-        const int mcnt = min(kMC, Nk - m0);
-        const double *Asrc = A + (size_t)m0 * rows3;
-        for (int i = tid; i < mcnt * rows3; i += kThreads) As[i] = Asrc[i];
-        if (tid < (1 + kRT) * kMC) {
-            const int mi = tid % kMC, side = tid / kMC;
-            double out[kG];
-            const int r = r0 + side - 1;
-            bool ok = mi < mcnt && (side == 0 || r < Rn);
-            double dist = (side == 0) ? chia : (ok ? R[r] * chia : 0.0);
-            if (ok && !real_ell) {
-                jl_group(kq[m0 + mi] * dist, lg, ng, out);
-            } else if (ok) {  // each non-integer multipole has its own recurrence
+    if (warp == kWork / 32) {
+        // ---------------------------------------------- A loader: blocks in the order of the MMAs
+        Ring ring;
+        uint32_t k = 0;
+        bool ok = true;
+        for (int win = 0; ok && win < nwin; win++)
+            for (int mt = 0; ok && mt < Mt; mt++)
+                for (int ks = 0; ks < kKS; ks++, k++, ring.next(kARing)) {
+                    const bool bad = !mbar_wait(&ctl->aempty[ring.st], ring.ph ^ 1, 32, kWaitLimit, abort_flag);
+                    if (__any_sync(0xffffffffu, bad)) {
+                        if (lane == 0) { atomicExch(err, 21); *abort_flag = 1; }
+                        ok = false;
+                        break;
+                    }
+                    if (elect_one()) {
+                        mbar_expect_tx(&ctl->afull[ring.st], kAStep);
+                        bulk_g2s(sA + (size_t)ring.st * kAStep,
+                                 dig + (((size_t)mt * nwin + win) * kKS + ks) * (kAStep / 16), kAStep,
+                                 &ctl->afull[ring.st]);
+                    }
+                    __syncwarp();
+                }
+        for (uint32_t h = (k > (uint32_t)kARing ? k - kARing : 0); h < k; h++)  // every load has landed before the exit
+            mbar_wait(&ctl->afull[h % kARing], (h / kARing) & 1, 32);
+        __syncwarp();
+    } else if (warp == kWork / 32 + 1) {
+        // ---------------------------------------------- MMA issuer
+        const uint32_t ab = __shfl_sync(0xffffffffu, smem_u32(sA), 0), bb = __shfl_sync(0xffffffffu, smem_u32(sB), 0);
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        Ring ring;
+        uint32_t fills = 0;  // accumulator fills so far
+        bool ok = true;
+        for (int win = 0; ok && win < nwin; win++)
+            for (int mt = 0; ok && mt < Mt; mt++, fills++)
+                for (int ks = 0; ks < kKS; ks++, ring.next(kARing)) {
+                    const bool bad =
+                        (ks == 0 && mt == 0 && !mbar_wait(&ctl->bready, win & 1, 32, kWaitLimit, abort_flag)) ||
+                        (ks == 0 && !mbar_wait(&ctl->dempty, (fills & 1) ^ 1, 32, kWaitLimit, abort_flag)) ||
+                        !mbar_wait(&ctl->afull[ring.st], ring.ph, 32, kWaitLimit, abort_flag);
+                    if (__any_sync(0xffffffffu, bad)) {
+                        if (lane == 0) { atomicExch(err, 22); *abort_flag = 1; }
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint64_t ad = sdesc_plain(ab + ring.st * kAStep, 128 * 16);
+                        const uint64_t bd = sdesc_plain(bb + ks * 2 * kRows * 16, kRows * 16);
 #pragma unroll
-                for (int g = 0; g < kG; g++) out[g] = (g < ng) ? jnu_real(lgr[g], kq[m0 + mi] * dist) : 0.0;
-            } else {
+                        for (int p = 0; p < 4; p++) {
+                            const int s = p < 2 ? p : p + 2;  // digit pairs (s, s + 2): levels from s on
+                            const uint32_t idesc = (1u << 4) | ((uint32_t)((kLev - s) * 16 >> 3) << 17) | (8u << 24);
 #pragma unroll
-                for (int g = 0; g < kG; g++) out[g] = 0.0;
+                            for (int cg = 0; cg < kCols / 16; cg++)
+                                umma_f16_ss(tm + cg * kRows + s * 16, ad + ((p * 2 * 128 * 16) >> 4),
+                                            bd + ((cg * kGroupBytes) >> 4), idesc, (ks | p) != 0);
+                        }
+                        umma_commit(&ctl->aempty[ring.st]);
+                        if (ks == kKS - 1) umma_commit(&ctl->dfull);
+                    }
+                    __syncwarp();
+                }
+        if (elect_one()) umma_commit(&ctl->mdone);  // every MMA has completed before TMEM is released
+        __syncwarp();
+        mbar_wait(&ctl->mdone, 0, 32);
+        __syncwarp();
+    } else {
+        // ---------------------------------------------- workers
+        const double chia = chi[a];
+        const int mi = tid % kMC, side = tid / kMC, rr = r0 + side - 1;  // chain: k node of the window, distance
+        const double dist = side == 0 ? chia : (side <= kRT && rr < Rn) ? R[rr] * chia : 0.0;
+        const int quad = warp & 3, cg = warp >> 2;  // TMEM lanes and column group taken out
+        uint32_t fills = 0;
+        bool dead = false;
+        auto take = [&](int win) {  // the window's sums join the output
+            for (int mt = 0; mt < Mt; mt++, fills++) {
+                if (!dead) {
+                    const bool bad = !mbar_wait(&ctl->dfull, fills & 1, 0, kWaitLimit, abort_flag);
+                    if (__any_sync(0xffffffffu, bad)) {
+                        if (lane == 0) { atomicExch(err, 23); *abort_flag = 1; }
+                        dead = true;
+                    }
+                }
+                if (dead) continue;
+                tc_fence_after();
+                const int row = mt * 128 + quad * 32 + lane;
+                const int me = ea[((size_t)mt * nwin + win) * 128 + quad * 32 + lane] - 994;
+                const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16) + cg * kRows;
+                const int t = row / N, n = row - t * N;
+#pragma unroll 1
+                for (int c4 = 0; c4 < 16; c4 += 4) {
+                    uint32_t D[kLev][4];
+#pragma unroll
+                    for (int l = 0; l < kLev; l++) tmem_ld4(tl + l * 16 + c4, D[l]);
+                    tmem_wait_ld4(D[0]);
+#pragma unroll
+                    for (int l = 1; l < kLev; l++) reg_fence4(D[l]);
+                    const int col = cg * 16 + c4, g = col / kRT, r = r0 + col % kRT;
+                    if (t < 3 && g < ng) {
+                        double *out = T + (((size_t)t * L + e0 + g) * N + n) * Q + (size_t)a * Rn + r;
+#pragma unroll
+                        for (int i = 0; i < 4; i++) {
+                            int d[kLev];
+#pragma unroll
+                            for (int l = 0; l < kLev; l++) {
+                                const float f = __uint_as_float(D[l][i]);
+                                d[l] = __float2int_rn(f + f);
+                            }
+                            const double v = fx_join(d, me + ctl->colmax[win & 1][col + i]);
+                            if (r + i < Rn) out[i] = win == 0 ? v : out[i] + v;
+                        }
+                    }
+                    __syncwarp();
+                }
+                tc_fence_before();
+                mbar_arrive(&ctl->dempty);
             }
+        };
+        for (int win = 0; win < nwin; win++) {
+            const int m0 = win * kMC, mcnt = min(kMC, Nk - m0);
+            if (side <= kRT) {
+                double *out = Jv + (side * kMC + mi) * kG;
+                const bool ok = !dead && mi < mcnt && dist > 0.0;
+                if (ok && !real_ell) {
+                    jl_group(kq[m0 + mi] * dist, ctl->lg, ng, out);
+                } else if (ok) {  // each non-integer multipole has its own recurrence
 #pragma unroll
-            for (int g = 0; g < kG; g++) Jv[tid * kG + g] = out[g];
-        }
-        __syncthreads();
-        for (int i = tid; i < kMC * kG * kRT; i += kThreads) {
-            const int mi = i / (kG * kRT), cmb = i % (kG * kRT);
-            const int g = cmb / kRT, rr = cmb % kRT;
-            Bp[i] = Jv[mi * kG + g] * Jv[((1 + rr) * kMC + mi) * kG + g];
-        }
-        __syncthreads();
-        for (int mi = 0; mi < mcnt; mi++) {
-            double b[kG];
+                    for (int g = 0; g < kG; g++) out[g] = (g < ng) ? jnu_real(ctl->lgr[g], kq[m0 + mi] * dist) : 0.0;
+                } else {
 #pragma unroll
-            for (int g = 0; g < kG; g++) b[g] = Bp[mi * kG * kRT + g * kRT + cb];
-#pragma unroll
-            for (int i = 0; i < ROWS; i++) {
-                const int row = rb + 32 * i;
-                const double av = (row < rows3) ? As[mi * rows3 + row] : 0.0;
-#pragma unroll
-                for (int g = 0; g < kG; g++) acc[i][g] = fma(av, b[g], acc[i][g]);
+                    for (int g = 0; g < kG; g++) out[g] = 0.0;
+                }
             }
+            if (tid < kCols) ctl->colmax[win & 1][tid] = 0;
+            if (win > 0) take(win - 1);  // its MMAs have read their digits
+            named_bar_sync(1, kWork);
+            // products j j of column (g, r) and of the k nodes of k-groups kg0 and kg0 + 8
+            const int col = tid % kCols, kg0 = tid / kCols, g = col / kRT, rc = col % kRT;
+            double p[2][4];
+            int mx = 0;
+#pragma unroll
+            for (int h = 0; h < 2; h++)
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    const int m = (kg0 + 8 * h) * 4 + i;
+                    p[h][i] = m < kMC ? Jv[m * kG + g] * Jv[((1 + rc) * kMC + m) * kG + g] : 0.0;
+                    mx = max(mx, (__double2hiint(p[h][i]) >> 20) & 0x7ff);
+                }
+            atomicMax(&ctl->colmax[win & 1][col], mx);
+            named_bar_sync(1, kWork);
+            const int M = ctl->colmax[win & 1][col];
+            const uint32_t top = fx_top(M < 70 ? kNone : M);
+            unsigned char *dst = sB + (col / 16) * kGroupBytes + (col % 16) * 16;
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int kg = kg0 + 8 * h;
+                if (kg >= kMC / 4) break;
+                uint64_t y[4];
+#pragma unroll
+                for (int i = 0; i < 4; i++) y[i] = fx_digits(p[h][i], top);
+                uint32_t prev[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};  // digits j - 2 and j - 1
+#pragma unroll
+                for (int j = 0; j < kLev; j++) {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        const uint32_t d =
+                            __half_as_ushort(__int2half_rn(((int)((y[i] >> (8 * (7 - j))) & 255) - 128) * 256));
+                        w[i] = (d << 16) | prev[0][i];
+                        prev[0][i] = prev[1][i];
+                        prev[1][i] = d;
+                    }
+                    *reinterpret_cast<uint4 *>(dst + (size_t)(kg * kRows + j * 16) * 16) =
+                        make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            }
+            fence_proxy_async();
+            mbar_arrive(&ctl->bready);
         }
-        __syncthreads();
+        take(nwin - 1);
     }
-    const int r = r0 + cb;
-    if (r >= Rn) return;
-#pragma unroll
-    for (int i = 0; i < ROWS; i++) {
-        const int row = rb + 32 * i;
-        if (row >= rows3) continue;
-        const int t = row / N, n = row % N;
-#pragma unroll
-        for (int g = 0; g < kG; g++) {
-            if (g >= ng) continue;
-            T[(((size_t)t * L + e0 + g) * N + n) * Q + (size_t)a * Rn + r] = acc[i][g];
-        }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == kWork / 32 + 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u));
     }
 }
 
@@ -313,35 +534,22 @@ __global__ void k_basis_to_f32(const double *__restrict__ T, float *__restrict__
     for (; i < n; i += stride) T32[i] = (float)T[i];
 }
 
-template <int ROWS>
-int launch_gemm_rows(blast_plan *p, const double *A, const double *kq, const double *ell, const double *R,
-                     cudaStream_t s)
-{
-    size_t smem = sizeof(double) * ((size_t)kMC * 3 * p->N + (size_t)(1 + kRT) * kMC * kG + (size_t)kMC * kG * kRT);
-    BL_CUDA(allow_opt_in_smem(k_basis_gemm<ROWS>, p->device));
-    dim3 grid((p->Rn + kRT - 1) / kRT, p->X);
-    for (int e0 = 0; e0 < p->L; e0 += kG) {
-        k_basis_gemm<ROWS><<<grid, kThreads, smem, s>>>(A, kq, p->Nk, p->N, ell, p->real_ell ? 1 : 0, p->L, e0,
-                                                        p->d_chi, R,
-                                                        p->Rn, p->Q, p->T64);
-        BL_CUDA(cudaGetLastError());
-    }
-    return BLAST_OK;
-}
-
 }  // namespace
 
 int launch_basis(blast_plan *p, cudaStream_t s)
 {
     const int rows3 = 3 * p->N;
-    if (rows3 > 32 * 12) return BLAST_EINVAL;  // n_cheb <= 128 (ROWS <= 12)
+    const int Mt = (rows3 + 127) / 128, nwin = (p->Nk + kMC - 1) / kMC;
+    uint4 *dig = nullptr;
+    uint16_t *ea = nullptr;
     double *kq = nullptr, *wq = nullptr, *A = nullptr, *R = nullptr;
     double *ell = nullptr;
     int rc = BLAST_OK;
     size_t nA = (size_t)p->Nk * rows3;
     if (cudaMalloc(&kq, sizeof(double) * p->Nk) || cudaMalloc(&wq, sizeof(double) * p->Nk) ||
         cudaMalloc(&A, sizeof(double) * nA) || cudaMalloc(&R, sizeof(double) * p->Rn) ||
-        cudaMalloc(&ell, sizeof(double) * p->L)) {
+        cudaMalloc(&ell, sizeof(double) * p->L) || cudaMalloc(&dig, (size_t)Mt * nwin * kKS * kAStep) ||
+        cudaMalloc(&ea, sizeof(uint16_t) * Mt * nwin * 128)) {
         cudaGetLastError();
         rc = BLAST_ENOMEM;
     }
@@ -355,14 +563,19 @@ int launch_basis(blast_plan *p, cudaStream_t s)
         if (cudaGetLastError() != cudaSuccess) rc = BLAST_EDEVICE;
     }
     if (!rc) {
-        int rows = (rows3 + 31) / 32;
-        if (rows <= 3) rc = launch_gemm_rows<3>(p, A, kq, ell, R, s);
-        else if (rows <= 6) rc = launch_gemm_rows<6>(p, A, kq, ell, R, s);
-        else if (rows <= 9) rc = launch_gemm_rows<9>(p, A, kq, ell, R, s);
-        else rc = launch_gemm_rows<12>(p, A, kq, ell, R, s);
+        k_basis_A_digits<<<dim3(nwin, Mt), 128, 0, s>>>(A, p->Nk, rows3, nwin, dig, ea);
+        const cudaError_t e0 = allow_opt_in_smem(k_basis_fx, p->device);
+        const dim3 grid((p->Rn + kRT - 1) / kRT, p->X, (p->L + kG - 1) / kG);
+        k_basis_fx<<<grid, kThreads, kBasisSmem, s>>>(dig, ea, Mt, nwin, kq, p->Nk, p->N, ell, p->real_ell ? 1 : 0, p->L,
+                                                      p->d_chi, R, p->Rn, p->Q, p->T64, p->d_err);
+        if (e0 != cudaSuccess || cudaGetLastError() != cudaSuccess) rc = BLAST_EDEVICE;
     }
     cudaStreamSynchronize(s);
-    cudaFree(kq); cudaFree(wq); cudaFree(A); cudaFree(R); cudaFree(ell);
+    cudaFree(kq); cudaFree(wq); cudaFree(A); cudaFree(R); cudaFree(ell); cudaFree(dig); cudaFree(ea);
+    if (!rc && *p->h_err) {  // a bounded wait gave up
+        *p->h_err = 0;
+        rc = BLAST_EDEVICE;
+    }
     if (!rc && cudaGetLastError() != cudaSuccess) rc = BLAST_EDEVICE;
     return rc;
 }
