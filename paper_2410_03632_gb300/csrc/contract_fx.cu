@@ -35,7 +35,7 @@
 //
 // Warp roles: TMA producer (FP64 basis tiles as they stand in memory, no
 // second table), MMA issuer, eight slicer warps (FP64 -> digits, integer and
-// half2 arithmetic), two epilogue warpgroups that take turns: while one joins
+// half2 arithmetic) with two warps that fetch the column exponents, two epilogue warpgroups that take turns: while one joins
 // levels (integer pipe) the other sums over R (FP64 pipe).
 //
 // What bounds it, and what it measured (64 ells, 128 x 128 nodes, order 64, 5+5
@@ -58,7 +58,7 @@ constexpr int kRows = kNB * kLev;        // rows of the coefficient operand, col
 constexpr int kM = 128;                  // chi-R nodes per tile
 constexpr int kKC = 32;                  // Chebyshev orders per chunk, in steps of 8 (one MMA K step)
 constexpr int kUnsigned = 76;            // largest n_cheb for unsigned basis digits
-constexpr int kThreads = 640;            // TMA, MMA, 2 spare, 8 epilogue and 8 slicer warps
+constexpr int kThreads = 640;            // TMA, MMA, 2 exponent, 8 epilogue and 8 slicer warps
 constexpr int kEpi0 = 4, kSli0 = 12;     // first epilogue and slicer warp
 constexpr int kWP = kM + 8;              // row pitch of w in shared memory (8 chains x 2 rows without conflicts)
 constexpr int kJC = 5;                   // tracers summed together
@@ -69,7 +69,11 @@ constexpr uint32_t kTmemCols = 512;              // two accumulators and the dig
 constexpr int kMaxRing = 4;
 constexpr int kBad = 1 << 20;            // exponent of coefficients that are not all finite
 
+constexpr int kTops = 4;                         // items whose column exponents are at hand
+
 struct FxCtl {
+    uint32_t top[kTops][kM];  // fx_top of the columns' exponents
+    uint64_t efull[kTops], eempty[kTops];
     uint64_t tfull[kMaxRing], tempty[kMaxRing], sfull[kChunks], sempty[kChunks], dfull[2], dempty[2], mdone;
     uint32_t tmem;
     int abort;
@@ -244,10 +248,12 @@ k_contract_fx(const __grid_constant__ CUtensorMap mapT, const FxArgs A)
     const int g = blockIdx.x % A.ngr, u0 = blockIdx.x / A.ngr, ustep = gridDim.x / A.ngr;
     const int b0 = g * A.gs, nbl = min(A.gs, A.n - b0);
     const int n_units = A.nqt * 3 * A.n_esel;
-    const FxItem first(A, u0, ustep, u0 < n_units ? (n_units - u0 + ustep - 1) / ustep : 0);
+    const int n_mine = u0 < n_units ? (n_units - u0 + ustep - 1) / ustep : 0, n_items = n_mine * A.rtq;
+    const FxItem first(A, u0, ustep, n_mine);
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < A.kT; i++) { mbar_init(&ctl->tfull[i], 1); mbar_init(&ctl->tempty[i], 4); }
+        for (int i = 0; i < kTops; i++) { mbar_init(&ctl->efull[i], 64); mbar_init(&ctl->eempty[i], 8); }
         for (int i = 0; i < kChunks; i++) { mbar_init(&ctl->sfull[i], 4); mbar_init(&ctl->sempty[i], 1); }
         for (int i = 0; i < 2; i++) { mbar_init(&ctl->dfull[i], 1); mbar_init(&ctl->dempty[i], 128); }
         mbar_init(&ctl->mdone, 1);
@@ -384,35 +390,43 @@ k_contract_fx(const __grid_constant__ CUtensorMap mapT, const FxArgs A)
         __syncwarp();
         mbar_wait(&ctl->mdone, 0, 32);
         __syncwarp();
+    } else if (warp < kEpi0) {
+        // ---------------------------------------------- column exponents, a few items ahead of the slicers:
+        // stepping through the items and the table's latency cost those a fifth of their time
+        Ring E;
+        const int q0 = (warp - 2) * 64 + lane;
+        for (FxItem it = first; !it.done(); it.next(A), E.next(kTops)) {
+            const FxPlace at(A, ctl->esel, it);
+            const uint16_t *row = A.cexp + at.slab(A) * A.Q + at.q0;
+            const int m0 = row[min(q0, at.cnt - 1)], m1 = row[min(q0 + 32, at.cnt - 1)];
+            const bool bad = !mbar_wait(&ctl->eempty[E.st], E.ph ^ 1, 0, kWaitLimit, abort_flag);
+            if (__any_sync(0xffffffffu, bad)) {
+                if (lane == 0) { atomicExch(A.err, 15); *abort_flag = 1; }
+                break;
+            }
+            ctl->top[E.st][q0] = fx_top(m0);
+            ctl->top[E.st][q0 + 32] = fx_top(m1);
+            mbar_arrive(&ctl->efull[E.st]);
+        }
     } else if (warp >= kSli0) {
         // ---------------------------------------------- slicers: two sets of four warps take every other chunk;
         // a thread owns one node (its TMEM lane), all orders of the chunk
         const int quad = warp & 3, q = quad * 32 + lane, set = (warp - kSli0) >> 2;
         const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + 2 * kRows;
-        Ring T, S;
+        Ring T, S, E;
         bool ok = true;
         int mine = set;  // chunks until the next one of this set
-        FxItem it = first, ahead = first;
-        auto col = [&]() -> int {  // exponent of this thread's column in the item ahead
-            if (ahead.done()) return kNone;
-            const FxPlace at(A, ctl->esel, ahead);
-            return A.cexp[at.slab(A) * A.Q + at.q0 + min(q, at.cnt - 1)];
-        };
-        // loaded two items ahead: the table comes from HBM
-        int m1 = col();
-        ahead.next(A);
-        int m2 = col();
-        for (; ok && !it.done(); it.next(A)) {
-            const uint32_t top = fx_top(m1);
-            m1 = m2;
-            ahead.next(A);
-            m2 = col();
+        for (int i = 0; ok && i < n_items; i++, E.next(kTops)) {
+            bool bad = !mbar_wait(&ctl->efull[E.st], E.ph, 0, kWaitLimit, abort_flag);
+            const uint32_t top = ctl->top[E.st][q];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->eempty[E.st]);
             for (int c = 0; c < nch; c++, T.next(A.kT), S.next(kChunks)) {
                 if (mine--) continue;
                 mine = 1;
                 const int ts = T.st, ss = S.st;
-                const bool bad = !mbar_wait(&ctl->tfull[ts], T.ph, 0, kWaitLimit, abort_flag) ||
-                                 !mbar_wait(&ctl->sempty[ss], S.ph ^ 1, 0, kWaitLimit, abort_flag);
+                bad = bad || !mbar_wait(&ctl->tfull[ts], T.ph, 0, kWaitLimit, abort_flag) ||
+                      !mbar_wait(&ctl->sempty[ss], S.ph ^ 1, 0, kWaitLimit, abort_flag);
                 if (__any_sync(0xffffffffu, bad)) {
                     if (lane == 0) { atomicExch(A.err, 13); *abort_flag = 1; }
                     ok = false;
