@@ -439,7 +439,7 @@ def run_blast(args):
         peak = peaks.get("hbm_gbs", 6800.0)
         achieved = alg_bytes / (avg_ms * 1e-3) / 1e9
         roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "peak_kind": "hbm copy, of measured", "traffic": traffic_for("eval.cu", "k_contract<float>", wl, B)}
+                "peak_kind": "hbm copy, of measured", "traffic": traffic_for("contract_f32.cu", "k_contract_f32", wl, B)}
     roof["kernel"] = kname
     roof["avg_launch_ms"] = avg_ms
     roof["launches"] = klaunch
@@ -460,10 +460,14 @@ def run_blast(args):
                           "unit": "GB/s"}
     cms, cl64 = prof_64["contract"]
     if cl64:
-        tf = method_flops / (cms / cl64 * 1e-3) / 1e12
+        # what the FP64 pipe is left with: the R sum's multiply-adds, one per chi-R node
+        # and B-side tracer of each type (the Chebyshev sum runs as exact digit products)
+        rsum_flops = sum(2.0 * sh[1] * plan.Q * (rq.n_clust + 2 * rq.n_lens) for sh, rq in zip(shapes, rqs))
+        tf = rsum_flops / (cms / cl64 * 1e-3) / 1e12
         kern["contract_fp64"] = {"bound": "alu", "achieved": tf, "peak": alu.get("fp64_tflops"),
                                  "frac": tf / alu["fp64_tflops"] if alu.get("fp64_tflops") else None,
-                                 "unit": "TFLOP/s", "peak_kind": "FP64 FMA, measured by the probe kernels"}
+                                 "unit": "TFLOP/s", "peak_kind": "FP64 FMA, measured by the probe kernels",
+                                 "flops_def": "2*(n_clust + 2 n_lens)*L*Q per cosmology (R sum)"}
 
     # single-request latency (p50 / p99) of the mixed path
     # the comparator of the serving numbers: requests one at a time in FP64
