@@ -676,7 +676,9 @@ int launch_contract_fx(blast_plan *p, const ReqDev *dreq, int n, const int *d_es
     const int optin = p->smem_optin, sms = p->sms;
     const size_t fixed = 128 + (size_t)nk8 * 2 * kRows * 16 + sizeof(double) * 2 * kNB * kWP + sizeof(FxCtl);
     A.kT = (int)(((size_t)optin - fixed) / kStageBytes);
-    if (A.kT > kMaxRing) A.kT = kMaxRing;
+    // even, so that a slot belongs to one set of slicers: with three, a set that comes back to
+    // a slot may find the phase of the other set's chunk still open and take it for its own
+    A.kT = A.kT >= kMaxRing ? kMaxRing : 2;
     const size_t smem = fixed + A.kT * kStageBytes;
 
     CUtensorMap map;
