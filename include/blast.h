@@ -61,7 +61,11 @@ typedef enum {
 /* Arithmetic of contraction (a) and quadrature (b).  The Chebyshev fit and the
  * basis precompute are always FP64. */
 typedef enum {
-    BLAST_FP64 = 0,   /* FP64 on CUDA cores (reference GPU path) */
+    BLAST_FP64 = 0,   /* FP64 results: the Chebyshev sum as exact products of
+                         eight base-256 digits per operand on FP16 tensor
+                         cores, joined with one rounding (FP64 multiply-adds
+                         for tables that the digits cannot hold); every other
+                         sum in FP64 multiply-adds */
     BLAST_FP32 = 1,   /* FP32 basis, FP32 CUDA-core contraction, FP64 final sums */
     BLAST_BF16S = 2   /* batched tcgen05 contraction on BF16 tensor cores: the
                          coefficients and each basis column are cut into five
@@ -168,7 +172,8 @@ int blast_plan_nodes(const blast_plan *plan, double *chi, double *R, double *k_c
 int blast_npairs(int n_clust, int n_lens);
 
 /* Step (pre), Eq. t_tilde: compute T~^{AB}_{n;l}(chi_a, R_r chi_a) for the
- * three types gg (f = k^2), gs (f = 1), ss (f = 1/k^2) in FP64 on the device,
+ * three types gg (f = k^2), gs (f = 1), ss (f = 1/k^2) in FP64 on the device
+ * (the k sum as exact digit products on the tensor cores, added in FP64),
  * then derive the copies named in precisions_mask (FP64 is always kept).
  * Synchronous with respect to the host when it returns.  Errors: BLAST_EDEVICE. */
 int blast_precompute_basis(blast_plan *plan, unsigned precisions_mask, void *stream);
@@ -370,8 +375,8 @@ int blast_graph_destroy(blast_graph *graph);
 /* Kernel classes of the evaluation path, for blast_profile_read. */
 #define BLAST_K_FIT 0         /* step (a0): Chebyshev fit */
 #define BLAST_K_WEIGHTS 1     /* quadrature weights U, V with growth folded in */
-#define BLAST_K_CONTRACT 2    /* steps (a) + (b, sum over R) on CUDA cores */
-#define BLAST_K_CONTRACT_TC 3 /* steps (a) + (b, sum over R) on tcgen05 tensor cores */
+#define BLAST_K_CONTRACT 2    /* steps (a) + (b, sum over R), FP64 and FP32 */
+#define BLAST_K_CONTRACT_TC 3 /* steps (a) + (b, sum over R), BF16 slices */
 #define BLAST_K_REDUCE 4      /* step (b, sum over chi) and prefactor */
 #define BLAST_K_CLASSES 5
 

@@ -35,13 +35,15 @@
 //
 // Warp roles: TMA producer (FP64 basis tiles as they stand in memory, no
 // second table), MMA issuer, eight slicer warps (FP64 -> digits, integer and
-// half2 arithmetic) with two warps that fetch the column exponents, two epilogue warpgroups that take turns: while one joins
-// levels (integer pipe) the other sums over R (FP64 pipe).
+// half2 arithmetic) with two warps that fetch the column exponents, two epilogue
+// warpgroups that take turns: while one joins levels (integer pipe) the other
+// sums over R (FP64 pipe).  Slicers that fetched the exponents themselves waited
+// for them (one cosmology 0.380 ms, with the two warps 0.365 ms).
 //
 // What bounds it, and what it measured (64 ells, 128 x 128 nodes, order 64, 5+5
 // tracers; the multiply-add kernel of eval.cu in brackets): one cosmology is
 // near the reading of the basis (1.61 GB: 0.24 ms) and bound by the slicers'
-// integer pipe, 0.38 ms (0.64 ms); 24 cosmologies 1.74 ms (14.0 ms), bound by
+// integer pipe, 0.37 ms (0.64 ms); 24 cosmologies 1.74 ms (14.0 ms), bound by
 // the FP64 multiply-adds of the R sum, five per node instead of 69, and by the
 // L2 latency of their weights.
 #include <cmath>

@@ -40,7 +40,11 @@ __device__ __forceinline__ void pair_decode(int p, int ng, int ns, int &t, int &
 }
 
 // ---------------------------------------------------------------------------
-// (a0) Chebyshev fit, one CTA per request.
+// (a0) Chebyshev fit, one CTA per request.  Bound by one SM's FP64 pipe (a warp
+// instruction holds a scheduler for 64 cycles: logarithms, reciprocals, sweeps)
+// and by the chain of dependent sweeps: 24 us for one request of 256 table
+// points at order 64 (37 us with every sweep run, two divisions a row in each
+// and the cosines read from L2).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kFitThreads)
 k_fit(ReqDev *reqs, int N, const double *__restrict__ node_u, const double *__restrict__ cos_tab)
@@ -236,7 +240,8 @@ k_contract(const ReqDev *__restrict__ reqs, const double *__restrict__ basis, in
 // type, selected ell), eight lanes a pair: lane c sums a = c, c + 8, .. and the
 // lanes meet in a tree, so the chain of a pair is X / 8 long (a thread per pair
 // waited for X loads and multiply-adds in turn: 36 us for one cosmology of
-// 5+5 tracers on 128 chi nodes and 64 ells, 88 us for 10+10 on 256 and 32).
+// 5+5 tracers on 128 chi nodes and 64 ells, now 11 us; 88 us for 10+10 on 256
+// and 32).
 //
 // sym: C_ij also gets N_AB(l) sum_a U_j(a) Y[t][es][a][i] (both kernel orders
 // of the symmetrised form, App. A); list positions are tracer rows minus the
