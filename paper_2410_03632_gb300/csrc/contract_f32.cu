@@ -75,8 +75,8 @@ k_contract_f32(const ReqDev *__restrict__ reqs, int n, const float *__restrict__
     extern __shared__ float4 sm4[];
     float *as = reinterpret_cast<float *>(sm4);  // [N][BB]
     float *red = as + (size_t)N * BB;            // [parity][tracer][v][BB]
-    constexpr int PB = (BB + 1) / 2;             // pairs of cosmologies (one of a single one is empty)
-    __shared__ __align__(16) int sV[3][2 * PB];  // a cosmology's list of a type, in floats from the first one's weights
+    constexpr int PB = BB / 2;                   // pairs of cosmologies
+    __shared__ __align__(16) int sV[3][BB];  // a cosmology's list of a type, in floats from the first one's weights
     __shared__ int sB[3][BB], sE[kSpan];
     __shared__ const float *sA[BB];
     const int g = blockIdx.x % ngr, rest = blockIdx.x / ngr, ntl = 3 * n_esel;
@@ -84,15 +84,15 @@ k_contract_f32(const ReqDev *__restrict__ reqs, int n, const float *__restrict__
     const int b0 = g * BB, nb = min(BB, n - b0), Q = X * Rn;
     const int tid = threadIdx.x, lane = tid & 31, pw = tid >> 5;
     const float *V0 = reqs[b0].V32 + (size_t)a * Rn;
-    if (tid < 2 * PB) {
+    if (tid < BB) {
         const bool live = tid < nb;
         const ReqDev &rq = reqs[b0 + (live ? tid : 0)];
         const int ng = rq.n_clust, ns = rq.n_lens, off = (int)(rq.V32 + (size_t)a * Rn - V0);
-        if (tid < BB) sA[tid] = rq.a32;
+        sA[tid] = rq.a32;
         for (int t = 0; t < 3; t++) {
             const bool both = sym && t == 1;
             sV[t][tid] = off + (t == 0 || both ? 0 : ng * Q);
-            if (tid < BB) sB[t][tid] = !live ? 0 : t == 0 ? ng : both ? ng + ns : ns;
+            sB[t][tid] = !live ? 0 : t == 0 ? ng : both ? ng + ns : ns;
         }
     }
     if (tid < kSpan && tl0 + tid < ntl) sE[tid] = esel[(tl0 + tid) % n_esel];
@@ -125,15 +125,11 @@ k_contract_f32(const ReqDev *__restrict__ reqs, int n, const float *__restrict__
                 const float x = __ldg(Tb + (size_t)k * Q + at[i]);
                 tv[i] = pair(x, x);
             }
-            if constexpr (BB % 4 == 0) {
 #pragma unroll
-                for (int b = 0; b < PB; b += 2) {
-                    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(as + (size_t)k * BB + 2 * b);
-                    av[b] = v.x;
-                    av[b + 1] = v.y;
-                }
-            } else {
-                av[0] = pair(as[k], 0.f);
+            for (int b = 0; b < PB; b += 2) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(as + (size_t)k * BB + 2 * b);
+                av[b] = v.x;
+                av[b + 1] = v.y;
             }
 #pragma unroll
             for (int b = 0; b < PB; b++)
@@ -150,7 +146,7 @@ k_contract_f32(const ReqDev *__restrict__ reqs, int n, const float *__restrict__
                 const int2 off = *reinterpret_cast<const int2 *>(&sV[t][2 * b]);
 #pragma unroll
                 for (int i = 0; i < NQ; i++)
-                    v[b][i] = pair(__ldg(Vj + (off.x + at[i])), BB > 1 ? __ldg(Vj + (off.y + at[i])) : 0.f);
+                    v[b][i] = pair(__ldg(Vj + (off.x + at[i])), __ldg(Vj + (off.y + at[i])));
             }
 #pragma unroll
             for (int p = 0; p < 2 && p < NQ; p++) {
@@ -198,20 +194,21 @@ int launch(blast_plan *p, const ReqDev *dreq, int n, const int *d_esel, int n_es
 
 }  // namespace
 
-// NQ R nodes a thread (64 NQ >= n_R); BB as many cosmologies as leave 32
-// accumulators, 4 for two to eight cosmologies (16 would multiply for empty
-// places), 1 for one.
+// NQ R nodes a thread (64 NQ >= n_R), BB cosmologies a block.  Places without a
+// cosmology are multiplied all the same, but a larger BB has more loads of the
+// basis in flight, so no grid has a variant for one cosmology: 128 R nodes of
+// order 64, one cosmology 0.31 ms with BB = 1, 0.29 with 4, 0.40 with 16; 192 of
+// order 96 1.04, 0.87 and (BB = 8) 0.70 ms.  Lines, in ms:
+//   NQ = 2, BB = 4 / 16: four cosmologies 0.32 / 0.42, eight 0.44 / 0.42 (on a
+//     grid of 16 ells and 64 x 64 nodes 0.028 / 0.035), twelve 0.57 / 0.42;
+//   NQ = 4, BB = 4 / 8: one 0.52 / 0.42, eight of order 96 1.38 / 0.80;
+//   NQ = 8, BB = 4 / 8: four 0.23 / 0.31 (320 nodes), 0.37 / 0.30 (512 nodes of
+//     order 96), eight 0.41 / 0.32 and 0.39 / 0.32.
 int launch_contract_f32(blast_plan *p, const ReqDev *dreq, int n, const int *d_esel, int n_esel, float *Y,
                         cudaStream_t s)
 {
-    const int nq = (p->Rn + 63) / 64;
-    if (nq <= 2)
-        return n == 1   ? launch<1, 2>(p, dreq, n, d_esel, n_esel, Y, s)
-               : n <= 8 ? launch<4, 2>(p, dreq, n, d_esel, n_esel, Y, s)
-                        : launch<16, 2>(p, dreq, n, d_esel, n_esel, Y, s);
-    if (nq <= 4)
-        return n == 1   ? launch<1, 4>(p, dreq, n, d_esel, n_esel, Y, s)
-               : n <= 4 ? launch<4, 4>(p, dreq, n, d_esel, n_esel, Y, s)
-                        : launch<8, 4>(p, dreq, n, d_esel, n_esel, Y, s);
-    return n == 1 ? launch<1, 8>(p, dreq, n, d_esel, n_esel, Y, s) : launch<4, 8>(p, dreq, n, d_esel, n_esel, Y, s);
+    if (p->Rn <= 128)
+        return n <= 8 ? launch<4, 2>(p, dreq, n, d_esel, n_esel, Y, s) : launch<16, 2>(p, dreq, n, d_esel, n_esel, Y, s);
+    if (p->Rn <= 256) return launch<8, 4>(p, dreq, n, d_esel, n_esel, Y, s);
+    return n <= 4 ? launch<4, 8>(p, dreq, n, d_esel, n_esel, Y, s) : launch<8, 8>(p, dreq, n, d_esel, n_esel, Y, s);
 }
