@@ -126,6 +126,15 @@ struct blast_plan {
     double prof_ms[BLAST_K_CLASSES] = {0};
 };
 
+// Work space of one request's weights U64, V64, U32, V32: every array and every
+// request starts on a multiple of 256 bytes.
+inline size_t request_weights_bytes(const blast_plan *p)
+{
+    const size_t ntr = p->max_clust + p->max_lens;
+    auto al = [](size_t b) { return (b + 255) / 256 * 256; };
+    return al(ntr * p->X * 8) + al(ntr * p->Q * 8) + al(ntr * p->X * 4) + al(ntr * p->Q * 4);
+}
+
 // Run one launcher under the plan's profiler: count it, and when timing is on
 // bracket it with events on stream s.
 template <class F> int prof_launch(blast_plan *p, int cls, cudaStream_t s, F &&fn)

@@ -21,6 +21,8 @@
 // one block per cosmology and node, which re-read the basis from L2 for each
 // and shuffled five times per tracer, took 19 ms; without the packed pairs and
 // the shared coefficients it was 1.22 ms.
+#include <climits>
+
 #include "blast_internal.h"
 
 namespace {
@@ -67,7 +69,11 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
     return d;
 }
 
-template <int BB, int NQ>
+// Off: type of an offset in floats from the weights of the block's first
+// cosmology.  The work spaces of a group span 45 (max_clust + max_lens) (n_chi + Q)
+// floats at BB = 16, past 2^31 from 1.5 million nodes of 16+16 tracers; 64-bit
+// offsets everywhere cost 2 % (48 cosmologies 1.28 ms a call instead of 1.26).
+template <int BB, int NQ, class Off>
 __global__ void __launch_bounds__(kThreads)
 k_contract_f32(const ReqDev *__restrict__ reqs, int n, const float *__restrict__ basis, int L, int N, int X, int Rn,
                const int *__restrict__ esel, int n_esel, int MT, int sym, int ngr, float *__restrict__ Y)
@@ -76,7 +82,8 @@ k_contract_f32(const ReqDev *__restrict__ reqs, int n, const float *__restrict__
     float *as = reinterpret_cast<float *>(sm4);  // [N][BB]
     float *red = as + (size_t)N * BB;            // [parity][tracer][v][BB]
     constexpr int PB = BB / 2;                   // pairs of cosmologies
-    __shared__ __align__(16) int sV[3][BB];  // a cosmology's list of a type, in floats from the first one's weights
+    struct alignas(2 * sizeof(Off)) Off2 { Off x, y; };
+    __shared__ __align__(16) Off sV[3][BB];  // a cosmology's list of a type, in floats from the first one's weights
     __shared__ int sB[3][BB], sE[kSpan];
     __shared__ const float *sA[BB];
     const int g = blockIdx.x % ngr, rest = blockIdx.x / ngr, ntl = 3 * n_esel;
@@ -87,11 +94,12 @@ k_contract_f32(const ReqDev *__restrict__ reqs, int n, const float *__restrict__
     if (tid < BB) {
         const bool live = tid < nb;
         const ReqDev &rq = reqs[b0 + (live ? tid : 0)];
-        const int ng = rq.n_clust, ns = rq.n_lens, off = (int)(rq.V32 + (size_t)a * Rn - V0);
+        const int ng = rq.n_clust, ns = rq.n_lens;
+        const Off off = (Off)(rq.V32 + (size_t)a * Rn - V0);
         sA[tid] = rq.a32;
         for (int t = 0; t < 3; t++) {
             const bool both = sym && t == 1;
-            sV[t][tid] = off + (t == 0 || both ? 0 : ng * Q);
+            sV[t][tid] = off + (t == 0 || both ? 0 : (Off)ng * Q);
             sB[t][tid] = !live ? 0 : t == 0 ? ng : both ? ng + ns : ns;
         }
     }
@@ -143,7 +151,7 @@ k_contract_f32(const ReqDev *__restrict__ reqs, int n, const float *__restrict__
             const float *Vj = V0 + (size_t)j * Q;
 #pragma unroll
             for (int b = 0; b < PB; b++) {
-                const int2 off = *reinterpret_cast<const int2 *>(&sV[t][2 * b]);
+                const Off2 off = *reinterpret_cast<const Off2 *>(&sV[t][2 * b]);
 #pragma unroll
                 for (int i = 0; i < NQ; i++)
                     v[b][i] = pair(__ldg(Vj + (off.x + at[i])), __ldg(Vj + (off.y + at[i])));
@@ -186,7 +194,9 @@ int launch(blast_plan *p, const ReqDev *dreq, int n, const int *d_esel, int n_es
     const int ngr = (n + BB - 1) / BB;
     const size_t smem = sizeof(float) * ((size_t)p->N * BB + (size_t)p->max_tr * 8 * BB);  // at most 24 KB
     const int nspan = (3 * n_esel + kSpan - 1) / kSpan;
-    k_contract_f32<BB, NQ><<<(unsigned)ngr * p->X * nspan, kThreads, smem, s>>>(
+    const bool near = request_weights_bytes(p) / sizeof(float) * BB <= INT_MAX;
+    (near ? k_contract_f32<BB, NQ, int> : k_contract_f32<BB, NQ, long long>)<<<(unsigned)ngr * p->X * nspan, kThreads,
+                                                                               smem, s>>>(
         dreq, n, p->T32, p->L, p->N, p->X, p->Rn, d_esel, n_esel, p->max_tr, p->r_form == 1, ngr, Y);
     BL_CUDA(cudaGetLastError());
     return BLAST_OK;

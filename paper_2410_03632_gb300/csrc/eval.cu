@@ -497,8 +497,8 @@ int stage_batch(blast_plan *p, int n, const blast_request *reqs, int prec, doubl
     size_t coef_per = al((size_t)p->N * 8) + al((size_t)p->N * 4) + al((size_t)kMaxPtab * 8);
     const size_t nl_per = al((size_t)p->L * p->X * 8);  // staged non-linear tables (host requests)
     size_t u64 = al((size_t)ntr_max * p->X * 8), v64 = al((size_t)ntr_max * p->Q * 8);
-    size_t u32 = al((size_t)ntr_max * p->X * 4), v32 = al((size_t)ntr_max * p->Q * 4);
-    size_t wts_per = u64 + v64 + u32 + v32;
+    size_t u32 = al((size_t)ntr_max * p->X * 4);
+    const size_t wts_per = request_weights_bytes(p);
     int pmax = blast_npairs(p->max_clust, p->max_lens);
     size_t cl_per = al((size_t)pmax * p->L * 8) / 8;
     int any_host_in = 0;
@@ -591,10 +591,8 @@ int stage_batch(blast_plan *p, int n, const blast_request *reqs, int prec, doubl
 int plan_reserve(blast_plan *p, int nmax, size_t *bytes)
 {
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-    const int ntr_max = p->max_clust + p->max_lens;
     const size_t coef_per = al((size_t)p->N * 8) + al((size_t)p->N * 4) + al((size_t)kMaxPtab * 8);
-    const size_t wts_per = al((size_t)ntr_max * p->X * 8) + al((size_t)ntr_max * p->Q * 8) +
-                           al((size_t)ntr_max * p->X * 4) + al((size_t)ntr_max * p->Q * 4);
+    const size_t wts_per = request_weights_bytes(p);
     size_t y = (size_t)nmax * 3 * p->L * p->X * p->max_tr * 8;  // CUDA-core partials (FP64)
     if (tc_supported(p)) y = std::max(y, tc_y_bytes(p, nmax, p->L));
     int rc;
