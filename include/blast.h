@@ -289,7 +289,9 @@ int blast_set_coef_envelope(blast_plan *plan, const double *env);
  *   returns   BLAST_ENOMEM when the request needs more scratch than the array
  *             holds (about 3 n_ell n_chi max_tracers + (n_clust+n_lens)
  *             n_chi n_R doubles; the 3x2pt 10+10-bin 100-ell grid fits),
- *             BLAST_ENOBASIS without an FP64 basis, BLAST_EDEVICE on CUDA errors.
+ *             BLAST_ENOBASIS without an FP64 basis, BLAST_EDEVICE on CUDA errors,
+ *             BLAST_ETIMEOUT (nothing launched) when a bounded device wait of an
+ *             earlier call on the plan gave up: that call's outputs are void
  * Set-up happens in blast_plan_create, on the plan's device with that device
  * current: it looks up the array's device address and loads the code of the
  * kernels this path launches (CUDA loads modules lazily), so the array's
@@ -392,7 +394,9 @@ int blast_profile_reset(blast_plan *plan);
 
 /* Test hook of the bounded device waits.  The next BLAST_BF16S call on the
  * plan has one epilogue warp of its first CTA wait, before tile `tile`, on a
- * barrier that nothing completes, with a limit of 2e7 clock cycles; the wait
+ * barrier that nothing completes, with a limit of 2e7 clock cycles (a BLAST_FP64
+ * call, blast_cl_noalloc included, if it comes first: the exponent warps of
+ * the contraction's first CTA, before its item `tile` or its last one); the wait
  * runs out, the kernel records the error word and every warp leaves after its
  * copies and MMAs in flight complete, and the call returns BLAST_ETIMEOUT (a
  * host-output call at once, a device-output call on the next call).  The

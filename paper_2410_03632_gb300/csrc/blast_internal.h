@@ -103,7 +103,7 @@ struct blast_plan {
     bool fx_ok = false;             // the digits of the FP64 tensor-core contraction hold this basis
     bool have64 = false, have32 = false, havebf = false;
     int *d_err = nullptr;           // host-mapped error word written by bounded device waits
-    int test_trip = -1;             // test hook of the tensor-core contraction (blast_test_trip_wait)
+    int test_trip = -1;             // test hook of the bounded waits (blast_test_trip_wait)
     int *h_err = nullptr;
     // side stream of a call: the Chebyshev fit runs there beside the weights
     // kernel (fork and join through the two events, in the caller's stream order)

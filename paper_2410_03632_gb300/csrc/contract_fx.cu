@@ -77,6 +77,7 @@ struct FxCtl {
     uint32_t top[kTops][kM];  // fx_top of the columns' exponents
     uint64_t efull[kTops], eempty[kTops];
     uint64_t tfull[kMaxRing], tempty[kMaxRing], sfull[kChunks], sempty[kChunks], dfull[2], dempty[2], mdone;
+    uint64_t never;  // no thread ever arrives on it (test hook)
     uint32_t tmem;
     int abort;
     const double *V[kNB];
@@ -99,6 +100,7 @@ struct FxArgs {
     const uint16_t *cexp;  // [3 L Q] biased exponent of the largest entry of a basis column
     double *Y;             // [n][3][n_esel][X][MT]
     int *err;
+    int trip;              // test hook: item before which CTA 0 waits on a barrier nothing completes (-1 off)
 };
 
 // MMA with A from tensor memory (128 lanes x 16 FP16 in 8 columns), B from shared memory.
@@ -259,6 +261,7 @@ k_contract_fx(const __grid_constant__ CUtensorMap mapT, const FxArgs A)
         for (int i = 0; i < kChunks; i++) { mbar_init(&ctl->sfull[i], 4); mbar_init(&ctl->sempty[i], 1); }
         for (int i = 0; i < 2; i++) { mbar_init(&ctl->dfull[i], 1); mbar_init(&ctl->dempty[i], 128); }
         mbar_init(&ctl->mdone, 1);
+        mbar_init(&ctl->never, 1);
         ctl->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -397,11 +400,13 @@ k_contract_fx(const __grid_constant__ CUtensorMap mapT, const FxArgs A)
         // stepping through the items and the table's latency cost those a fifth of their time
         Ring E;
         const int q0 = (warp - 2) * 64 + lane;
-        for (FxItem it = first; !it.done(); it.next(A), E.next(kTops)) {
+        int trip = blockIdx.x == 0 ? min(A.trip, n_items - 1) : -1;  // items until the test hook's wait
+        for (FxItem it = first; !it.done(); it.next(A), E.next(kTops), trip--) {
             const FxPlace at(A, ctl->esel, it);
             const uint16_t *row = A.cexp + at.slab(A) * A.Q + at.q0;
             const int m0 = row[min(q0, at.cnt - 1)], m1 = row[min(q0 + 32, at.cnt - 1)];
-            const bool bad = !mbar_wait(&ctl->eempty[E.st], E.ph ^ 1, 0, kWaitLimit, abort_flag);
+            const bool bad = (trip == 0 && !mbar_wait(&ctl->never, 0, 32, kTripLimit, abort_flag)) ||
+                             !mbar_wait(&ctl->eempty[E.st], E.ph ^ 1, 0, kWaitLimit, abort_flag);
             if (__any_sync(0xffffffffu, bad)) {
                 if (lane == 0) { atomicExch(A.err, 15); *abort_flag = 1; }
                 break;
@@ -676,6 +681,8 @@ int launch_contract_fx(blast_plan *p, const ReqDev *dreq, int n, const int *d_es
     A.cexp = p->colexp;
     A.Y = Y;
     A.err = p->d_err;
+    A.trip = p->test_trip;
+    p->test_trip = -1;  // one call only
     const int nk8 = (A.N + 7) / 8;
     const int optin = p->smem_optin, sms = p->sms;
     const size_t fixed = 128 + (size_t)nk8 * 2 * kRows * 16 + sizeof(double) * 2 * kNB * kWP + sizeof(FxCtl);

@@ -628,10 +628,10 @@ k_contract_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ 
                     const int buf = g % kNBUF;
                     if (!dead) {
                         bool lost = *abort_flag != 0;
-                        // test hook: one warp of CTA 0 waits, with a 20M-cycle limit, on a
+                        // test hook: one warp of CTA 0 waits, with a short limit, on a
                         // barrier nothing completes, so the bounded wait runs out
                         if (!lost && (int)g == args.trip && blockIdx.x == 0 && quad % nqb == 0 &&
-                            !mbar_wait(never, 0, 0, 20000000LL)) {
+                            !mbar_wait(never, 0, 0, kTripLimit)) {
                             lost = true;
                             atomicExch(args.err, 4);
                             *abort_flag = 1;

@@ -124,6 +124,10 @@ extern "C" int blast_cl_noalloc(blast_plan *p, const blast_request *r, double *c
         return BLAST_ENOMEM;
     }
     if (!p->have64) return BLAST_ENOBASIS;
+    if (*p->h_err) {  // a bounded device wait of an earlier call gave up
+        *p->h_err = 0;
+        return BLAST_ETIMEOUT;
+    }
 
     if (cudaSetDevice(p->device) != cudaSuccess) { cudaGetLastError(); return BLAST_EDEVICE; }
     unsigned char *S = nullptr;

@@ -9,6 +9,7 @@
 namespace {
 
 constexpr long long kWaitLimit = 4000000000LL;  // clock cycles (about 2 s)
+constexpr long long kTripLimit = 20000000LL;    // clock cycles of the test hook's wait
 constexpr uint32_t kSuspendNs = 1000000;        // longest suspension of one phase test
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
