@@ -175,7 +175,10 @@ int blast_npairs(int n_clust, int n_lens);
  * three types gg (f = k^2), gs (f = 1), ss (f = 1/k^2) in FP64 on the device
  * (the k sum as exact digit products on the tensor cores, added in FP64),
  * then derive the copies named in precisions_mask (FP64 is always kept).
- * Synchronous with respect to the host when it returns.  Errors: BLAST_EDEVICE. */
+ * Synchronous with respect to the host when it returns.  Errors: BLAST_ENOMEM,
+ * BLAST_EDEVICE, BLAST_ETIMEOUT (a bounded wait of the build itself gave up; the
+ * plan has no basis then.  A wait of an earlier call is left for the next
+ * evaluation to report). */
 int blast_precompute_basis(blast_plan *plan, unsigned precisions_mask, void *stream);
 
 /* Copy the FP64 basis between the plan and a caller buffer of
@@ -396,7 +399,9 @@ int blast_profile_reset(blast_plan *plan);
  * plan has one epilogue warp of its first CTA wait, before tile `tile`, on a
  * barrier that nothing completes, with a limit of 2e7 clock cycles (a BLAST_FP64
  * call, blast_cl_noalloc included, if it comes first: the exponent warps of
- * the contraction's first CTA, before its item `tile` or its last one); the wait
+ * the contraction's first CTA, before its item `tile` or its last one;
+ * blast_precompute_basis: the first CTA's loader, at k window `tile` or the
+ * last); the wait
  * runs out, the kernel records the error word and every warp leaves after its
  * copies and MMAs in flight complete, and the call returns BLAST_ETIMEOUT (a
  * host-output call at once, a device-output call on the next call).  The

@@ -39,6 +39,7 @@ constexpr int kARing = 3;
 
 struct BasisCtl {
     uint64_t afull[kARing], aempty[kARing], bready, dfull, dempty, mdone;
+    uint64_t never;  // no thread ever arrives on it (test hook)
     uint32_t tmem;
     int abort;
     int colmax[2][kCols];  // biased exponent of a column's largest entry, by parity of the window
@@ -303,7 +304,8 @@ __device__ __forceinline__ void umma_f16_ss(uint32_t d_tmem, uint64_t ad, uint64
 __global__ void __launch_bounds__(kThreads, 1)
 k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int Mt, int nwin,
            const double *__restrict__ kq, int Nk, int N, const double *__restrict__ ell, int real_ell, int L,
-           const double *__restrict__ chi, const double *__restrict__ R, int Rn, int Q, double *__restrict__ T, int *err)
+           const double *__restrict__ chi, const double *__restrict__ R, int Rn, int Q, double *__restrict__ T, int *err,
+           int trip)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *sB = (unsigned char *)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);  // [group][k-group][row][16 B]
@@ -320,6 +322,7 @@ k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int M
         mbar_init(&ctl->dfull, 1);
         mbar_init(&ctl->dempty, kWork);
         mbar_init(&ctl->mdone, 1);
+        mbar_init(&ctl->never, 1);
         ctl->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -341,11 +344,13 @@ k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int M
         // ---------------------------------------------- A loader: blocks in the order of the MMAs
         Ring ring;
         uint32_t k = 0;
+        const int stop = blockIdx.x + blockIdx.y + blockIdx.z == 0 ? min(trip, nwin - 1) : -1;  // test hook's window
         bool ok = true;
         for (int win = 0; ok && win < nwin; win++)
             for (int mt = 0; ok && mt < Mt; mt++)
                 for (int ks = 0; ks < kKS; ks++, k++, ring.next(kARing)) {
-                    const bool bad = !mbar_wait(&ctl->aempty[ring.st], ring.ph ^ 1, 32, kWaitLimit, abort_flag);
+                    const bool bad = (win == stop && !mbar_wait(&ctl->never, 0, 32, kTripLimit, abort_flag)) ||
+                                     !mbar_wait(&ctl->aempty[ring.st], ring.ph ^ 1, 32, kWaitLimit, abort_flag);
                     if (__any_sync(0xffffffffu, bad)) {
                         if (lane == 0) { atomicExch(err, 21); *abort_flag = 1; }
                         ok = false;
@@ -544,19 +549,23 @@ int launch_basis(blast_plan *p, cudaStream_t s)
     uint16_t *ea = nullptr;
     double *kq = nullptr, *wq = nullptr, *A = nullptr, *R = nullptr;
     double *ell = nullptr;
+    int *err = nullptr, gave_up = 0;  // the build's own error word: the plan's may hold an earlier call's
+    const int trip = p->test_trip;
+    p->test_trip = -1;  // one call only
     int rc = BLAST_OK;
     size_t nA = (size_t)p->Nk * rows3;
     if (cudaMalloc(&kq, sizeof(double) * p->Nk) || cudaMalloc(&wq, sizeof(double) * p->Nk) ||
         cudaMalloc(&A, sizeof(double) * nA) || cudaMalloc(&R, sizeof(double) * p->Rn) ||
         cudaMalloc(&ell, sizeof(double) * p->L) || cudaMalloc(&dig, (size_t)Mt * nwin * kKS * kAStep) ||
-        cudaMalloc(&ea, sizeof(uint16_t) * Mt * nwin * 128)) {
+        cudaMalloc(&ea, sizeof(uint16_t) * Mt * nwin * 128) || cudaMalloc(&err, sizeof(int))) {
         cudaGetLastError();
         rc = BLAST_ENOMEM;
     }
     if (!rc && (cudaMemcpyAsync(kq, p->kq.data(), sizeof(double) * p->Nk, cudaMemcpyHostToDevice, s) ||
                 cudaMemcpyAsync(wq, p->wq.data(), sizeof(double) * p->Nk, cudaMemcpyHostToDevice, s) ||
                 cudaMemcpyAsync(R, p->R.data(), sizeof(double) * p->Rn, cudaMemcpyHostToDevice, s) ||
-                cudaMemcpyAsync(ell, p->ell.data(), sizeof(double) * p->L, cudaMemcpyHostToDevice, s)))
+                cudaMemcpyAsync(ell, p->ell.data(), sizeof(double) * p->L, cudaMemcpyHostToDevice, s) ||
+                cudaMemsetAsync(err, 0, sizeof(int), s)))
         rc = BLAST_EDEVICE;
     if (!rc) {
         k_basis_A<<<(p->Nk + 255) / 256, 256, 0, s>>>(kq, wq, p->Nk, p->N, p->kmap, p->k_min, p->k_max, A);
@@ -567,15 +576,14 @@ int launch_basis(blast_plan *p, cudaStream_t s)
         const cudaError_t e0 = allow_opt_in_smem(k_basis_fx, p->device);
         const dim3 grid((p->Rn + kRT - 1) / kRT, p->X, (p->L + kG - 1) / kG);
         k_basis_fx<<<grid, kThreads, kBasisSmem, s>>>(dig, ea, Mt, nwin, kq, p->Nk, p->N, ell, p->real_ell ? 1 : 0, p->L,
-                                                      p->d_chi, R, p->Rn, p->Q, p->T64, p->d_err);
-        if (e0 != cudaSuccess || cudaGetLastError() != cudaSuccess) rc = BLAST_EDEVICE;
+                                                      p->d_chi, R, p->Rn, p->Q, p->T64, err, trip);
+        if (e0 != cudaSuccess || cudaGetLastError() != cudaSuccess ||
+            cudaMemcpyAsync(&gave_up, err, sizeof(int), cudaMemcpyDeviceToHost, s))
+            rc = BLAST_EDEVICE;
     }
-    cudaStreamSynchronize(s);
-    cudaFree(kq); cudaFree(wq); cudaFree(A); cudaFree(R); cudaFree(ell); cudaFree(dig); cudaFree(ea);
-    if (!rc && *p->h_err) {  // a bounded wait gave up
-        *p->h_err = 0;
-        rc = BLAST_EDEVICE;
-    }
+    if (cudaStreamSynchronize(s) != cudaSuccess && !rc) rc = BLAST_EDEVICE;
+    cudaFree(kq); cudaFree(wq); cudaFree(A); cudaFree(R); cudaFree(ell); cudaFree(dig); cudaFree(ea); cudaFree(err);
+    if (!rc && gave_up) rc = BLAST_ETIMEOUT;
     if (!rc && cudaGetLastError() != cudaSuccess) rc = BLAST_EDEVICE;
     return rc;
 }

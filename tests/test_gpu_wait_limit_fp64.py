@@ -1,4 +1,5 @@
-"""The bounded waits of the FP64 tensor-core contraction, made to run out.
+"""The bounded waits of the FP64 tensor-core contraction and of the basis
+integrals, made to run out.
 
 The test hook has two warps of the first CTA wait on a barrier that nothing
 completes, with a short limit.  The kernel records its error word and leaves
@@ -71,3 +72,39 @@ def test_noalloc_reports_the_call_before(plan):
     out.fill_(float("nan"))
     assert call() == bl.BLAST_OK
     assert torch.equal(out, ref)
+
+
+def test_basis_build(plan):
+    ref = plan.basis()
+    chi, R, _ = plan.nodes()
+    rq = synth.config_request("tc", chi, R, 0)
+    for window in (0, 7):
+        assert bl.blast_test_trip_wait(plan.h, window) == bl.BLAST_OK
+        with pytest.raises(bl.BlastError) as ei:
+            plan.precompute(bl.BLAST_BASIS_FP64)
+        assert ei.value.status == bl.BLAST_ETIMEOUT
+        with pytest.raises(bl.BlastError) as ei:
+            plan.cl(rq, bl.BLAST_FP64)
+        assert ei.value.status == bl.BLAST_ENOBASIS
+        plan.precompute(bl.BLAST_BASIS_FP64)
+        np.testing.assert_array_equal(plan.basis(), ref)
+
+
+def test_basis_build_after_a_call_that_gave_up(plan):
+    """The build succeeds, and the earlier call's failure is reported by the next evaluation."""
+    import torch
+
+    ref = plan.basis()
+    chi, R, _ = plan.nodes()
+    rq = synth.config_request("tc", chi, R, 0)
+    want = plan.cl(rq, bl.BLAST_FP64)
+    out = torch.empty(want.shape, dtype=torch.float64, device="cuda")
+    assert bl.blast_test_trip_wait(plan.h, 0) == bl.BLAST_OK
+    assert bl.blast_cl(plan.h, plan.request(rq), bl.BLAST_FP64, out.data_ptr(), 1, None) == bl.BLAST_OK
+    torch.cuda.synchronize()
+    plan.precompute(bl.BLAST_BASIS_FP64)
+    np.testing.assert_array_equal(plan.basis(), ref)
+    with pytest.raises(bl.BlastError) as ei:
+        plan.cl(rq, bl.BLAST_FP64)
+    assert ei.value.status == bl.BLAST_ETIMEOUT
+    np.testing.assert_array_equal(plan.cl(rq, bl.BLAST_FP64), want)
