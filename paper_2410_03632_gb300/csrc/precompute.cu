@@ -8,15 +8,22 @@
 //
 // The GEMM runs as exact integer products on the FP16 tensor cores (eight 8-bit
 // digits an operand, eight exact levels; contract_fx.cu states the arithmetic),
-// over windows of 56 k nodes: in a window every row of A and every column of B
-// has its own exponent, the window's sum is exact in the levels up to the
-// dropped ones (2^-59 of its largest product), and windows add in FP64.  What is
+// over windows of at most 56 k nodes: in a window every row of A and every column
+// of B has its own exponent, the window's sum is exact in the levels up to the
+// dropped ones (about 2^-58 of the row's largest entry times the column's), and
+// windows add in FP64.  The two largest entries can lie at different nodes (1/k^2
+// falls where j_l j_l rises), so a window also ends where w_m, w_m k^2 or w_m / k^2
+// has varied by more than 2^6: what is dropped then stays under 2^-52 of the
+// window's largest product up to T_n.  Few nodes on a wide k range need it (k over
+// [1e-4, 10], 17 nodes, l = 2, type ss: 7e-11 of the sum of magnitudes with one
+// window, 1.5e-16 with five); 65,537 nodes get 1172 windows instead of 1171.  What is
 // left on the FP64 pipe (two multiply-adds a clock and SM) are the recurrences,
 // a product per entry of B and an addition per output and window.
 //
 // Bound by the recurrences.  16 ells to 200, 38 x 64 nodes, order 32, 65,537 k
 // nodes: 0.31 s (with the GEMM in FP64 multiply-adds and 2l + 1 counted up in
 // FP64 0.81 s); error against an independent FP64 evaluation 2e-15 (9e-15).
+#include <algorithm>
 #include <cmath>
 
 #include "blast_internal.h"
@@ -27,7 +34,8 @@ namespace {
 
 constexpr int kG = 8;     // plan ells per CTA (one group)
 constexpr int kRT = 8;    // R nodes per CTA
-constexpr int kMC = 56;   // k nodes per window: (1 + kRT) * kMC = 504 Bessel chains
+constexpr int kMC = 56;   // most k nodes of a window: (1 + kRT) * kMC = 504 Bessel chains
+constexpr double kSpread = 64.0;  // largest spread of the quadrature's factors in a window
 constexpr int kKS = kMC / 8;              // MMA K steps of a window (8 k nodes, two digits each)
 constexpr int kWork = 512;                // worker threads; then the A loader and the MMA issuer
 constexpr int kThreads = kWork + 64;
@@ -261,14 +269,14 @@ __device__ double jnu_real(double nu, double x)
 // its own exponent in a window; the layout is the MMA operand's, one 16 KB block
 // per (row tile, window, K step).
 __global__ void __launch_bounds__(128)
-k_basis_A_digits(const double *__restrict__ A, int Nk, int rows3, int nwin, uint4 *__restrict__ dig,
-                 uint16_t *__restrict__ ea)
+k_basis_A_digits(const double *__restrict__ A, const int *__restrict__ wstart, int rows3, int nwin,
+                 uint4 *__restrict__ dig, uint16_t *__restrict__ ea)
 {
-    const int win = blockIdx.x, mt = blockIdx.y, row = mt * 128 + threadIdx.x, m0 = win * kMC;
+    const int win = blockIdx.x, mt = blockIdx.y, row = mt * 128 + threadIdx.x, m0 = wstart[win], m1 = wstart[win + 1];
     const bool live = row < rows3;
     int mx = 0;
     for (int i = 0; i < kMC; i++)
-        if (live && m0 + i < Nk) mx = max(mx, (__double2hiint(A[(size_t)(m0 + i) * rows3 + row]) >> 20) & 0x7ff);
+        if (live && m0 + i < m1) mx = max(mx, (__double2hiint(A[(size_t)(m0 + i) * rows3 + row]) >> 20) & 0x7ff);
     const int M = mx < 70 ? kNone : mx;
     ea[((size_t)mt * nwin + win) * 128 + threadIdx.x] = (uint16_t)M;
     const uint32_t top = fx_top(M);
@@ -278,7 +286,7 @@ k_basis_A_digits(const double *__restrict__ A, int Nk, int rows3, int nwin, uint
 #pragma unroll
         for (int i = 0; i < 4; i++) {
             const int m = m0 + kg * 4 + i;
-            fx_pairs<false>(live && m < Nk ? A[(size_t)m * rows3 + row] : 0.0, top, w[0][i], w[1][i], w[2][i], w[3][i]);
+            fx_pairs<false>(live && m < m1 ? A[(size_t)m * rows3 + row] : 0.0, top, w[0][i], w[1][i], w[2][i], w[3][i]);
         }
 #pragma unroll
         for (int p = 0; p < 4; p++)
@@ -303,7 +311,7 @@ __device__ __forceinline__ void umma_f16_ss(uint32_t d_tmem, uint64_t ad, uint64
 // products j j for the MMAs, which run beside the next window's recurrences.
 __global__ void __launch_bounds__(kThreads, 1)
 k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int Mt, int nwin,
-           const double *__restrict__ kq, int Nk, int N, const double *__restrict__ ell, int real_ell, int L,
+           const double *__restrict__ kq, const int *__restrict__ wstart, int N, const double *__restrict__ ell, int real_ell, int L,
            const double *__restrict__ chi, const double *__restrict__ R, int Rn, int Q, double *__restrict__ T, int *err,
            int trip)
 {
@@ -460,8 +468,9 @@ k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int M
                 mbar_arrive(&ctl->dempty);
             }
         };
+        int m0 = 0, m1 = wstart[1];  // the window's nodes; the next one's end is fetched a window ahead
         for (int win = 0; win < nwin; win++) {
-            const int m0 = win * kMC, mcnt = min(kMC, Nk - m0);
+            const int m2 = wstart[min(win + 2, nwin)], mcnt = m1 - m0;
             if (side <= kRT) {
                 double *out = Jv + (side * kMC + mi) * kG;
                 const bool ok = !dead && mi < mcnt && dist > 0.0;
@@ -520,6 +529,8 @@ k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int M
             }
             fence_proxy_async();
             mbar_arrive(&ctl->bready);
+            m0 = m1;
+            m1 = m2;
         }
         take(nwin - 1);
     }
@@ -539,16 +550,38 @@ __global__ void k_basis_to_f32(const double *__restrict__ T, float *__restrict__
     for (; i < n; i += stride) T32[i] = (float)T[i];
 }
 
+// First k nodes of the windows, and the end.
+std::vector<int> k_windows(const std::vector<double> &k, const std::vector<double> &w)
+{
+    const int n = (int)k.size();
+    std::vector<int> start(1, 0);
+    double lo[3], hi[3];
+    for (int m = 0; m < n; m++) {
+        const double f[3] = {w[m] * k[m] * k[m], w[m], w[m] / (k[m] * k[m])};
+        bool fits = m > 0 && m - start.back() < kMC;
+        for (int i = 0; i < 3 && fits; i++) fits = std::max(hi[i], f[i]) <= kSpread * std::min(lo[i], f[i]);
+        if (m > 0 && !fits) start.push_back(m);
+        for (int i = 0; i < 3; i++) {
+            lo[i] = fits ? std::min(lo[i], f[i]) : f[i];
+            hi[i] = fits ? std::max(hi[i], f[i]) : f[i];
+        }
+    }
+    start.push_back(n);
+    return start;
+}
+
 }  // namespace
 
 int launch_basis(blast_plan *p, cudaStream_t s)
 {
     const int rows3 = 3 * p->N;
-    const int Mt = (rows3 + 127) / 128, nwin = (p->Nk + kMC - 1) / kMC;
+    const std::vector<int> wstart = k_windows(p->kq, p->wq);
+    const int Mt = (rows3 + 127) / 128, nwin = (int)wstart.size() - 1;
     uint4 *dig = nullptr;
     uint16_t *ea = nullptr;
     double *kq = nullptr, *wq = nullptr, *A = nullptr, *R = nullptr;
     double *ell = nullptr;
+    int *ws = nullptr;
     int *err = nullptr, gave_up = 0;  // the build's own error word: the plan's may hold an earlier call's
     const int trip = p->test_trip;
     p->test_trip = -1;  // one call only
@@ -557,7 +590,8 @@ int launch_basis(blast_plan *p, cudaStream_t s)
     if (cudaMalloc(&kq, sizeof(double) * p->Nk) || cudaMalloc(&wq, sizeof(double) * p->Nk) ||
         cudaMalloc(&A, sizeof(double) * nA) || cudaMalloc(&R, sizeof(double) * p->Rn) ||
         cudaMalloc(&ell, sizeof(double) * p->L) || cudaMalloc(&dig, (size_t)Mt * nwin * kKS * kAStep) ||
-        cudaMalloc(&ea, sizeof(uint16_t) * Mt * nwin * 128) || cudaMalloc(&err, sizeof(int))) {
+        cudaMalloc(&ea, sizeof(uint16_t) * Mt * nwin * 128) || cudaMalloc(&ws, sizeof(int) * wstart.size()) ||
+        cudaMalloc(&err, sizeof(int))) {
         cudaGetLastError();
         rc = BLAST_ENOMEM;
     }
@@ -565,6 +599,7 @@ int launch_basis(blast_plan *p, cudaStream_t s)
                 cudaMemcpyAsync(wq, p->wq.data(), sizeof(double) * p->Nk, cudaMemcpyHostToDevice, s) ||
                 cudaMemcpyAsync(R, p->R.data(), sizeof(double) * p->Rn, cudaMemcpyHostToDevice, s) ||
                 cudaMemcpyAsync(ell, p->ell.data(), sizeof(double) * p->L, cudaMemcpyHostToDevice, s) ||
+                cudaMemcpyAsync(ws, wstart.data(), sizeof(int) * wstart.size(), cudaMemcpyHostToDevice, s) ||
                 cudaMemsetAsync(err, 0, sizeof(int), s)))
         rc = BLAST_EDEVICE;
     if (!rc) {
@@ -572,17 +607,18 @@ int launch_basis(blast_plan *p, cudaStream_t s)
         if (cudaGetLastError() != cudaSuccess) rc = BLAST_EDEVICE;
     }
     if (!rc) {
-        k_basis_A_digits<<<dim3(nwin, Mt), 128, 0, s>>>(A, p->Nk, rows3, nwin, dig, ea);
+        k_basis_A_digits<<<dim3(nwin, Mt), 128, 0, s>>>(A, ws, rows3, nwin, dig, ea);
         const cudaError_t e0 = allow_opt_in_smem(k_basis_fx, p->device);
         const dim3 grid((p->Rn + kRT - 1) / kRT, p->X, (p->L + kG - 1) / kG);
-        k_basis_fx<<<grid, kThreads, kBasisSmem, s>>>(dig, ea, Mt, nwin, kq, p->Nk, p->N, ell, p->real_ell ? 1 : 0, p->L,
+        k_basis_fx<<<grid, kThreads, kBasisSmem, s>>>(dig, ea, Mt, nwin, kq, ws, p->N, ell, p->real_ell ? 1 : 0, p->L,
                                                       p->d_chi, R, p->Rn, p->Q, p->T64, err, trip);
         if (e0 != cudaSuccess || cudaGetLastError() != cudaSuccess ||
             cudaMemcpyAsync(&gave_up, err, sizeof(int), cudaMemcpyDeviceToHost, s))
             rc = BLAST_EDEVICE;
     }
     if (cudaStreamSynchronize(s) != cudaSuccess && !rc) rc = BLAST_EDEVICE;
-    cudaFree(kq); cudaFree(wq); cudaFree(A); cudaFree(R); cudaFree(ell); cudaFree(dig); cudaFree(ea); cudaFree(err);
+    cudaFree(kq); cudaFree(wq); cudaFree(A); cudaFree(R); cudaFree(ell); cudaFree(dig); cudaFree(ea); cudaFree(ws);
+    cudaFree(err);
     if (!rc && gave_up) rc = BLAST_ETIMEOUT;
     if (!rc && cudaGetLastError() != cudaSuccess) rc = BLAST_EDEVICE;
     return rc;
