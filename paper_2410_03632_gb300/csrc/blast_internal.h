@@ -80,6 +80,7 @@ struct blast_plan {
     // host grids
     std::vector<double> chi, wchi, R, wR, tcheb, kcheb;
     std::vector<double> kq, wq;  // Clenshaw-Curtis nodes / weights in k
+    std::vector<int> kwin;       // windows of the basis build: their first k nodes, and the end
     uint64_t grid_hash = 0;
 
     // device constant tables
@@ -171,6 +172,7 @@ struct ReqDev {
 
 // Launchers (defined in the kernel translation units) ------------------------
 int launch_basis(blast_plan *p, cudaStream_t s);
+std::vector<int> basis_windows(const std::vector<double> &k, const std::vector<double> &w);
 int launch_basis_convert(blast_plan *p, unsigned mask, cudaStream_t s);
 int launch_fit(blast_plan *p, ReqDev *dreq, int nreq, cudaStream_t s);
 int launch_weights(blast_plan *p, ReqDev *dreq, int nreq, int want32, cudaStream_t s, int want_v64 = 1);

@@ -282,6 +282,7 @@ extern "C" int blast_plan_create(const blast_plan_desc *d, blast_plan **out)
     p->kq.resize(nq + 1);
     p->wq.resize(nq + 1);
     for (int m = 0; m <= nq; m++) { p->kq[m] = kc + kh * cx[m]; p->wq[m] = kh * cw[m]; }
+    p->kwin = basis_windows(p->kq, p->wq);
 
     // grid hash (for basis files)
     uint64_t hsh = fnv1a(p->ell.data(), sizeof(double) * p->L);

@@ -12,11 +12,11 @@
 // of B has its own exponent, the window's sum is exact in the levels up to the
 // dropped ones (about 2^-58 of the row's largest entry times the column's), and
 // windows add in FP64.  The two largest entries can lie at different nodes (1/k^2
-// falls where j_l j_l rises), so a window also ends where w_m, w_m k^2 or w_m / k^2
-// has varied by more than 2^6: what is dropped then stays under 2^-52 of the
+// falls where j_l j_l rises), so a window also ends where the spreads of w_m and k^2
+// multiply to more than 2^6: what is dropped then stays under 2^-52 of the
 // window's largest product up to T_n.  Few nodes on a wide k range need it (k over
 // [1e-4, 10], 17 nodes, l = 2, type ss: 7e-11 of the sum of magnitudes with one
-// window, 1.5e-16 with five); 65,537 nodes get 1172 windows instead of 1171.  What is
+// window, 1.5e-16 with five); 65,537 nodes get 1173 windows instead of 1171.  What is
 // left on the FP64 pipe (two multiply-adds a clock and SM) are the recurrences,
 // a product per entry of B and an addition per output and window.
 //
@@ -35,7 +35,7 @@ namespace {
 constexpr int kG = 8;     // plan ells per CTA (one group)
 constexpr int kRT = 8;    // R nodes per CTA
 constexpr int kMC = 56;   // most k nodes of a window: (1 + kRT) * kMC = 504 Bessel chains
-constexpr double kSpread = 64.0;  // largest spread of the quadrature's factors in a window
+constexpr double kSpread = 64.0;  // largest product of the spreads of w_m and k^2 in a window
 constexpr int kKS = kMC / 8;              // MMA K steps of a window (8 k nodes, two digits each)
 constexpr int kWork = 512;                // worker threads; then the A loader and the MMA issuer
 constexpr int kThreads = kWork + 64;
@@ -44,6 +44,7 @@ constexpr int kRows = 16 * kLev;          // rows of a column group's operand, T
 constexpr uint32_t kGroupBytes = (kMC / 4) * kRows * 16;  // a column group's digits: [k-group of 4][row][16 B]
 constexpr uint32_t kAStep = 4 * 2 * 128 * 16;  // A's digits of a K step: [pair][k-group][128 rows][16 B]
 constexpr int kARing = 3;
+constexpr size_t kPartBytes = (size_t)256 << 20;  // digits of A in memory at a time
 
 struct BasisCtl {
     uint64_t afull[kARing], aempty[kARing], bready, dfull, dempty, mdone;
@@ -267,12 +268,14 @@ __device__ double jnu_real(double nu, double x)
 
 // Digits of A: rows t N + n of 128-row tiles, window by window, each row with
 // its own exponent in a window; the layout is the MMA operand's, one 16 KB block
-// per (row tile, window, K step).
+// per (row tile, window, K step).  wstart lists the part's windows, A starts at its
+// first node.
 __global__ void __launch_bounds__(128)
 k_basis_A_digits(const double *__restrict__ A, const int *__restrict__ wstart, int rows3, int nwin,
                  uint4 *__restrict__ dig, uint16_t *__restrict__ ea)
 {
-    const int win = blockIdx.x, mt = blockIdx.y, row = mt * 128 + threadIdx.x, m0 = wstart[win], m1 = wstart[win + 1];
+    const int win = blockIdx.x, mt = blockIdx.y, row = mt * 128 + threadIdx.x;
+    const int m0 = wstart[win] - wstart[0], m1 = wstart[win + 1] - wstart[0];
     const bool live = row < rows3;
     int mx = 0;
     for (int i = 0; i < kMC; i++)
@@ -309,11 +312,12 @@ __device__ __forceinline__ void umma_f16_ss(uint32_t d_tmem, uint64_t ad, uint64
 // 128-row tiles of A in turn.  Per window the workers run the recurrences, then
 // take the previous window's sums out of TMEM, then write the digits of the
 // products j j for the MMAs, which run beside the next window's recurrences.
+// A launch takes the windows of one part of the k nodes; all but the first add to T.
 __global__ void __launch_bounds__(kThreads, 1)
 k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int Mt, int nwin,
-           const double *__restrict__ kq, const int *__restrict__ wstart, int N, const double *__restrict__ ell, int real_ell, int L,
-           const double *__restrict__ chi, const double *__restrict__ R, int Rn, int Q, double *__restrict__ T, int *err,
-           int trip)
+           const double *__restrict__ kq, const int *__restrict__ wstart, int add, int N,
+           const double *__restrict__ ell, int real_ell, int L, const double *__restrict__ chi,
+           const double *__restrict__ R, int Rn, int Q, double *__restrict__ T, int *err, int trip)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *sB = (unsigned char *)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);  // [group][k-group][row][16 B]
@@ -459,7 +463,7 @@ k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int M
                                 d[l] = __float2int_rn(f + f);
                             }
                             const double v = fx_join(d, me + ctl->colmax[win & 1][col + i]);
-                            if (r + i < Rn) out[i] = win == 0 ? v : out[i] + v;
+                            if (r + i < Rn) out[i] = add | win ? out[i] + v : v;
                         }
                     }
                     __syncwarp();
@@ -468,17 +472,22 @@ k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int M
                 mbar_arrive(&ctl->dempty);
             }
         };
-        int m0 = 0, m1 = wstart[1];  // the window's nodes; the next one's end is fetched a window ahead
+        // the window's nodes and this chain's k; the next ones are fetched a window ahead
+        int m0 = wstart[0], m1 = wstart[1];
+        const int kend = wstart[nwin] - 1;
+        double kx = kq[min(m0 + mi, kend)];
         for (int win = 0; win < nwin; win++) {
             const int m2 = wstart[min(win + 2, nwin)], mcnt = m1 - m0;
+            const double k = kx;
+            kx = kq[min(m1 + mi, kend)];
             if (side <= kRT) {
                 double *out = Jv + (side * kMC + mi) * kG;
                 const bool ok = !dead && mi < mcnt && dist > 0.0;
                 if (ok && !real_ell) {
-                    jl_group(kq[m0 + mi] * dist, ctl->lg, ng, out);
+                    jl_group(k * dist, ctl->lg, ng, out);
                 } else if (ok) {  // each non-integer multipole has its own recurrence
 #pragma unroll
-                    for (int g = 0; g < kG; g++) out[g] = (g < ng) ? jnu_real(ctl->lgr[g], kq[m0 + mi] * dist) : 0.0;
+                    for (int g = 0; g < kG; g++) out[g] = (g < ng) ? jnu_real(ctl->lgr[g], k * dist) : 0.0;
                 } else {
 #pragma unroll
                     for (int g = 0; g < kG; g++) out[g] = 0.0;
@@ -550,50 +559,63 @@ __global__ void k_basis_to_f32(const double *__restrict__ T, float *__restrict__
     for (; i < n; i += stride) T32[i] = (float)T[i];
 }
 
-// First k nodes of the windows, and the end.
-std::vector<int> k_windows(const std::vector<double> &k, const std::vector<double> &w)
+}  // namespace
+
+std::vector<int> basis_windows(const std::vector<double> &k, const std::vector<double> &w)
 {
     const int n = (int)k.size();
     std::vector<int> start(1, 0);
-    double lo[3], hi[3];
-    for (int m = 0; m < n; m++) {
-        const double f[3] = {w[m] * k[m] * k[m], w[m], w[m] / (k[m] * k[m])};
-        bool fits = m > 0 && m - start.back() < kMC;
-        for (int i = 0; i < 3 && fits; i++) fits = std::max(hi[i], f[i]) <= kSpread * std::min(lo[i], f[i]);
-        if (m > 0 && !fits) start.push_back(m);
-        for (int i = 0; i < 3; i++) {
-            lo[i] = fits ? std::min(lo[i], f[i]) : f[i];
-            hi[i] = fits ? std::max(hi[i], f[i]) : f[i];
+    double lo = w[0], hi = w[0], k0 = k[0] * k[0];  // k falls
+    for (int m = 1, first = 0; m < n; m++) {
+        const double l = std::min(lo, w[m]), h = std::max(hi, w[m]);
+        if (m - first < kMC && h * k0 <= kSpread * l * (k[m] * k[m])) {
+            lo = l;
+            hi = h;
+        } else {
+            start.push_back(first = m);
+            lo = hi = w[m];
+            k0 = k[m] * k[m];
         }
     }
     start.push_back(n);
     return start;
 }
 
-}  // namespace
-
 int launch_basis(blast_plan *p, cudaStream_t s)
 {
     const int rows3 = 3 * p->N;
-    const std::vector<int> wstart = k_windows(p->kq, p->wq);
+    const std::vector<int> &wstart = p->kwin;
     const int Mt = (rows3 + 127) / 128, nwin = (int)wstart.size() - 1;
     uint4 *dig = nullptr;
     uint16_t *ea = nullptr;
-    double *kq = nullptr, *wq = nullptr, *A = nullptr, *R = nullptr;
-    double *ell = nullptr;
-    int *ws = nullptr;
-    int *err = nullptr, gave_up = 0;  // the build's own error word: the plan's may hold an earlier call's
+    double *A = nullptr, *tab = nullptr;
+    int gave_up = 0;
     const int trip = p->test_trip;
     p->test_trip = -1;  // one call only
     int rc = BLAST_OK;
-    size_t nA = (size_t)p->Nk * rows3;
-    if (cudaMalloc(&kq, sizeof(double) * p->Nk) || cudaMalloc(&wq, sizeof(double) * p->Nk) ||
-        cudaMalloc(&A, sizeof(double) * nA) || cudaMalloc(&R, sizeof(double) * p->Rn) ||
-        cudaMalloc(&ell, sizeof(double) * p->L) || cudaMalloc(&dig, (size_t)Mt * nwin * kKS * kAStep) ||
-        cudaMalloc(&ea, sizeof(uint16_t) * Mt * nwin * 128) || cudaMalloc(&ws, sizeof(int) * wstart.size()) ||
-        cudaMalloc(&err, sizeof(int))) {
+    const size_t ntab = 2 * (size_t)p->Nk + p->Rn + p->L;
+    if (cudaMalloc(&tab, sizeof(double) * ntab + sizeof(int) * (wstart.size() + 1))) {
         cudaGetLastError();
-        rc = BLAST_ENOMEM;
+        return BLAST_ENOMEM;
+    }
+    double *kq = tab, *wq = kq + p->Nk, *R = wq + p->Nk, *ell = R + p->Rn;
+    int *ws = reinterpret_cast<int *>(tab + ntab);
+    int *err = ws + wstart.size();  // the build's own error word: the plan's may hold an earlier call's
+    // A and its digits take three times (rows padded to 128: up to 43 times) the memory of A
+    // alone, so they are made for a part of the windows at a time, and for smaller parts
+    // where even that is not to be had.  The sums do not depend on the parts.
+    const size_t wbytes = (size_t)Mt * kKS * kAStep;
+    const int parts = (int)((nwin * wbytes + kPartBytes - 1) / kPartBytes);
+    int per = (nwin + parts - 1) / parts;  // windows of a part
+    while (!rc) {
+        if (!cudaMalloc(&A, sizeof(double) * per * kMC * rows3) && !cudaMalloc(&dig, per * wbytes) &&
+            !cudaMalloc(&ea, sizeof(uint16_t) * Mt * per * 128))
+            break;
+        cudaGetLastError();
+        cudaFree(A); cudaFree(dig); cudaFree(ea);
+        A = nullptr; dig = nullptr; ea = nullptr;
+        if (per == 1) rc = BLAST_ENOMEM;
+        per = (per + 1) / 2;
     }
     if (!rc && (cudaMemcpyAsync(kq, p->kq.data(), sizeof(double) * p->Nk, cudaMemcpyHostToDevice, s) ||
                 cudaMemcpyAsync(wq, p->wq.data(), sizeof(double) * p->Nk, cudaMemcpyHostToDevice, s) ||
@@ -602,23 +624,21 @@ int launch_basis(blast_plan *p, cudaStream_t s)
                 cudaMemcpyAsync(ws, wstart.data(), sizeof(int) * wstart.size(), cudaMemcpyHostToDevice, s) ||
                 cudaMemsetAsync(err, 0, sizeof(int), s)))
         rc = BLAST_EDEVICE;
-    if (!rc) {
-        k_basis_A<<<(p->Nk + 255) / 256, 256, 0, s>>>(kq, wq, p->Nk, p->N, p->kmap, p->k_min, p->k_max, A);
+    if (!rc && allow_opt_in_smem(k_basis_fx, p->device) != cudaSuccess) rc = BLAST_EDEVICE;
+    for (int w0 = 0; w0 < nwin && !rc; w0 += per) {
+        const int nw = std::min(per, nwin - w0), m0 = wstart[w0], nk = wstart[w0 + nw] - m0;
+        k_basis_A<<<(nk + 255) / 256, 256, 0, s>>>(kq + m0, wq + m0, nk, p->N, p->kmap, p->k_min, p->k_max, A);
+        if (cudaGetLastError() != cudaSuccess) rc = BLAST_EDEVICE;
+        k_basis_A_digits<<<dim3(nw, Mt), 128, 0, s>>>(A, ws + w0, rows3, nw, dig, ea);
+        const dim3 grid((p->Rn + kRT - 1) / kRT, p->X, (p->L + kG - 1) / kG);
+        k_basis_fx<<<grid, kThreads, kBasisSmem, s>>>(dig, ea, Mt, nw, kq, ws + w0, w0 > 0, p->N, ell,
+                                                      p->real_ell ? 1 : 0, p->L, p->d_chi, R, p->Rn, p->Q, p->T64, err,
+                                                      w0 ? -1 : trip);
         if (cudaGetLastError() != cudaSuccess) rc = BLAST_EDEVICE;
     }
-    if (!rc) {
-        k_basis_A_digits<<<dim3(nwin, Mt), 128, 0, s>>>(A, ws, rows3, nwin, dig, ea);
-        const cudaError_t e0 = allow_opt_in_smem(k_basis_fx, p->device);
-        const dim3 grid((p->Rn + kRT - 1) / kRT, p->X, (p->L + kG - 1) / kG);
-        k_basis_fx<<<grid, kThreads, kBasisSmem, s>>>(dig, ea, Mt, nwin, kq, ws, p->N, ell, p->real_ell ? 1 : 0, p->L,
-                                                      p->d_chi, R, p->Rn, p->Q, p->T64, err, trip);
-        if (e0 != cudaSuccess || cudaGetLastError() != cudaSuccess ||
-            cudaMemcpyAsync(&gave_up, err, sizeof(int), cudaMemcpyDeviceToHost, s))
-            rc = BLAST_EDEVICE;
-    }
+    if (!rc && cudaMemcpyAsync(&gave_up, err, sizeof(int), cudaMemcpyDeviceToHost, s)) rc = BLAST_EDEVICE;
     if (cudaStreamSynchronize(s) != cudaSuccess && !rc) rc = BLAST_EDEVICE;
-    cudaFree(kq); cudaFree(wq); cudaFree(A); cudaFree(R); cudaFree(ell); cudaFree(dig); cudaFree(ea); cudaFree(ws);
-    cudaFree(err);
+    cudaFree(tab); cudaFree(A); cudaFree(dig); cudaFree(ea);
     if (!rc && gave_up) rc = BLAST_ETIMEOUT;
     if (!rc && cudaGetLastError() != cudaSuccess) rc = BLAST_EDEVICE;
     return rc;

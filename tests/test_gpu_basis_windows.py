@@ -52,3 +52,39 @@ def test_few_nodes(nk, chi_lo, chi_hi):
             size = (w * k ** float(p)) @ (_envelope(l, k[:, None] * c1) * _envelope(l, k[:, None] * c2))
             err = np.max(np.abs(T[t, e] - ref[t, e]) / size)
             assert err < 1e-14, (t, l, err)
+
+
+def test_many_nodes_take_bounded_memory():
+    """The digits are made part by part (four here): the build holds less than the FP64 A[k node][3 N]
+    alone would take (403 MB).  The k sum has 131,073 terms, sqrt(131073) 2^-54 = 2e-14 for a chain of
+    random roundings: 1e-13 of the sum of magnitudes."""
+    import threading
+    import time
+
+    import torch
+
+    N, nk = 128, 2 ** 17 + 1
+    ells = np.array([2, 40], np.int32)
+    spec = synth.PlanSpec(ells, 4, 300.0, 4100.0, 2, 0.5, 1.5, N, 1e-4, 10.0, 1, nk, 1, 1)
+    plan = bl.Plan(spec)
+    plan.precompute(bl.BLAST_BASIS_FP64)    # tables and code are in place
+    T = plan.basis()
+    free0, done, least = torch.cuda.mem_get_info()[0], threading.Event(), []
+    worker = threading.Thread(target=lambda: (plan.precompute(bl.BLAST_BASIS_FP64), done.set()))
+    worker.start()
+    while not done.is_set():
+        least.append(torch.cuda.mem_get_info()[0])
+        time.sleep(1e-3)
+    worker.join()
+    np.testing.assert_array_equal(plan.basis(), T)
+    plan.close()
+    took = free0 - min(least)
+    assert 0 < took < 24 * N * nk, took
+    g = orc.Grid(ells, 4, 300.0, 4100.0, 2, 0.5, 1.5, N, 1e-4, 10.0, nk, 1)
+    ref = g.basis().reshape(T.shape)
+    k, _, w = orc.cc_grid(nk, 1e-4, 10.0)
+    c1, c2 = np.repeat(g.chi, 2), (g.chi[:, None] * g.R).ravel()
+    for t, p in enumerate((2, 0, -2)):
+        for e, l in enumerate(ells):
+            size = (w * k ** float(p)) @ (_envelope(l, k[:, None] * c1) * _envelope(l, k[:, None] * c2))
+            assert np.max(np.abs(T[t, e, :4] - ref[t, e, :4]) / size) < 1e-13, (t, l)
