@@ -317,7 +317,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int Mt, int nwin,
            const double *__restrict__ kq, const int *__restrict__ wstart, int add, int N,
            const double *__restrict__ ell, int real_ell, int L, const double *__restrict__ chi,
-           const double *__restrict__ R, int Rn, int Q, double *__restrict__ T, int *err, int trip)
+           const double *__restrict__ R, int Rn, int Q, double *__restrict__ T, int *err,
+           long long limit, int trip)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *sB = (unsigned char *)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);  // [group][k-group][row][16 B]
@@ -362,7 +363,7 @@ k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int M
             for (int mt = 0; ok && mt < Mt; mt++)
                 for (int ks = 0; ks < kKS; ks++, k++, ring.next(kARing)) {
                     const bool bad = (win == stop && !mbar_wait(&ctl->never, 0, 32, kTripLimit, abort_flag)) ||
-                                     !mbar_wait(&ctl->aempty[ring.st], ring.ph ^ 1, 32, kWaitLimit, abort_flag);
+                                     !mbar_wait(&ctl->aempty[ring.st], ring.ph ^ 1, 32, limit, abort_flag);
                     if (__any_sync(0xffffffffu, bad)) {
                         if (lane == 0) { atomicExch(err, 21); *abort_flag = 1; }
                         ok = false;
@@ -390,9 +391,9 @@ k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int M
             for (int mt = 0; ok && mt < Mt; mt++, fills++)
                 for (int ks = 0; ks < kKS; ks++, ring.next(kARing)) {
                     const bool bad =
-                        (ks == 0 && mt == 0 && !mbar_wait(&ctl->bready, win & 1, 32, kWaitLimit, abort_flag)) ||
-                        (ks == 0 && !mbar_wait(&ctl->dempty, (fills & 1) ^ 1, 32, kWaitLimit, abort_flag)) ||
-                        !mbar_wait(&ctl->afull[ring.st], ring.ph, 32, kWaitLimit, abort_flag);
+                        (ks == 0 && mt == 0 && !mbar_wait(&ctl->bready, win & 1, 32, limit, abort_flag)) ||
+                        (ks == 0 && !mbar_wait(&ctl->dempty, (fills & 1) ^ 1, 32, limit, abort_flag)) ||
+                        !mbar_wait(&ctl->afull[ring.st], ring.ph, 32, limit, abort_flag);
                     if (__any_sync(0xffffffffu, bad)) {
                         if (lane == 0) { atomicExch(err, 22); *abort_flag = 1; }
                         ok = false;
@@ -431,7 +432,7 @@ k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int M
         auto take = [&](int win) {  // the window's sums join the output
             for (int mt = 0; mt < Mt; mt++, fills++) {
                 if (!dead) {
-                    const bool bad = !mbar_wait(&ctl->dfull, fills & 1, 0, kWaitLimit, abort_flag);
+                    const bool bad = !mbar_wait(&ctl->dfull, fills & 1, 0, limit, abort_flag);
                     if (__any_sync(0xffffffffu, bad)) {
                         if (lane == 0) { atomicExch(err, 23); *abort_flag = 1; }
                         dead = true;
@@ -624,6 +625,13 @@ int launch_basis(blast_plan *p, cudaStream_t s)
                 cudaMemcpyAsync(ws, wstart.data(), sizeof(int) * wstart.size(), cudaMemcpyHostToDevice, s) ||
                 cudaMemsetAsync(err, 0, sizeof(int), s)))
         rc = BLAST_EDEVICE;
+    // The waits cover the recurrences of a window, 512 chains at two FP64 lanes a clock: an
+    // operation of every chain takes 256 cycles, a step about 14 of them with a division,
+    // real orders have a recurrence each, and a warp may run both directions.  Eight times
+    // that: a full window of eight real multipoles near 1e5 takes 4e9 cycles, where a fixed
+    // limit of 4e9 ran out.
+    const double top = p->ell.back(), steps = (top + 20.0 + 10.0 * cbrt(top)) * (p->real_ell ? kG : 1);
+    const long long limit = kWaitLimit + (long long)(steps * (8 * 2 * 14 * 256));
     if (!rc && allow_opt_in_smem(k_basis_fx, p->device) != cudaSuccess) rc = BLAST_EDEVICE;
     for (int w0 = 0; w0 < nwin && !rc; w0 += per) {
         const int nw = std::min(per, nwin - w0), m0 = wstart[w0], nk = wstart[w0 + nw] - m0;
@@ -633,7 +641,7 @@ int launch_basis(blast_plan *p, cudaStream_t s)
         const dim3 grid((p->Rn + kRT - 1) / kRT, p->X, (p->L + kG - 1) / kG);
         k_basis_fx<<<grid, kThreads, kBasisSmem, s>>>(dig, ea, Mt, nw, kq, ws + w0, w0 > 0, p->N, ell,
                                                       p->real_ell ? 1 : 0, p->L, p->d_chi, R, p->Rn, p->Q, p->T64, err,
-                                                      w0 ? -1 : trip);
+                                                      limit, w0 ? -1 : trip);
         if (cudaGetLastError() != cudaSuccess) rc = BLAST_EDEVICE;
     }
     if (!rc && cudaMemcpyAsync(&gave_up, err, sizeof(int), cudaMemcpyDeviceToHost, s)) rc = BLAST_EDEVICE;
