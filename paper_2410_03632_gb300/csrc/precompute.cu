@@ -18,7 +18,9 @@
 // [1e-4, 10], 17 nodes, l = 2, type ss: 7e-11 of the sum of magnitudes with one
 // window, 1.5e-16 with five); 65,537 nodes get 1173 windows instead of 1171.  What is
 // left on the FP64 pipe (two multiply-adds a clock and SM) are the recurrences,
-// a product per entry of B and an addition per output and window.
+// a product per entry of B and an addition per output and window.  Infinities and
+// NaN (the integer recurrences leave the FP64 range below x of about 1e-24) make
+// their integrals NaN; entries under 2^-953 count as zero.
 //
 // Bound by the recurrences.  16 ells to 200, 38 x 64 nodes, order 32, 65,537 k
 // nodes: 0.31 s (with the GEMM in FP64 multiply-adds and 2l + 1 counted up in
@@ -463,7 +465,10 @@ k_basis_fx(const uint4 *__restrict__ dig, const uint16_t *__restrict__ ea, int M
                                 const float f = __uint_as_float(D[l][i]);
                                 d[l] = __float2int_rn(f + f);
                             }
-                            const double v = fx_join(d, me + ctl->colmax[win & 1][col + i]);
+                            const int mc = ctl->colmax[win & 1][col + i];
+                            double v = fx_join(d, me + mc);
+                            // an infinity or NaN has no digits: the sum is what a product with it is
+                            if (mc == 2047 || me == 2047 - 994) v = __longlong_as_double(0x7ff8000000000000ll);
                             if (r + i < Rn) out[i] = add | win ? out[i] + v : v;
                         }
                     }

@@ -88,3 +88,16 @@ def test_many_nodes_take_bounded_memory():
         for e, l in enumerate(ells):
             size = (w * k ** float(p)) @ (_envelope(l, k[:, None] * c1) * _envelope(l, k[:, None] * c2))
             assert np.max(np.abs(T[t, e, :4] - ref[t, e, :4]) / size) < 1e-13, (t, l)
+
+
+def test_recurrences_out_of_range_are_not_numbers():
+    """At distances of 1e-24 the downward recurrence of l = 40's group overflows: those integrals are NaN,
+    the others (chi^4 k^5 and less: 1e-88) stay what they are, and no made-up number stands between."""
+    spec = synth.PlanSpec(np.array([2, 3, 40], np.int32), 4, 1e-24, 4e-24, 4, 0.5, 1.5, 3, 1e-2, 10.0, 1, 65, 1, 1)
+    plan = bl.Plan(spec)
+    plan.precompute(bl.BLAST_BASIS_FP64)
+    T = plan.basis()
+    plan.close()
+    bad = np.isnan(T)
+    assert bad.any() and not bad.all()
+    assert np.all(np.abs(T[~bad]) < 1e-60)
