@@ -65,7 +65,11 @@ typedef enum {
                          eight base-256 digits per operand on FP16 tensor
                          cores, joined with one rounding (FP64 multiply-adds
                          for tables that the digits cannot hold); every other
-                         sum in FP64 multiply-adds */
+                         sum in FP64 multiply-adds.  The Chebyshev sum's error is
+                         about 2^-59 max_n |a_n| max_n |T~_n| (n_cheb 2^-56 of it
+                         at most), not relative to its largest term; the rounding
+                         of the a_n in the fit, 2^-53 max_n |a_n| each, moves it
+                         by more */
     BLAST_FP32 = 1,   /* FP32 basis, FP32 CUDA-core contraction, FP64 final sums */
     BLAST_BF16S = 2   /* batched tcgen05 contraction on BF16 tensor cores: the
                          coefficients and each basis column are cut into five

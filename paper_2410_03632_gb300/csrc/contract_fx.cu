@@ -14,10 +14,17 @@
 // |digit| <= 128 (64 for p = 0).  A digit is exact in FP16, a product below
 // 2^14, and level k, D_k = sum_{p+q=k} sum_n a_p t_q, below 2^24 for n_cheb <=
 // 128 and k <= 7, so the FP32 accumulation of levels 0..7 is exact in any
-// order.  The dropped levels are under 2^-53 of n_cheb times the largest
-// product in the worst case and about 2^-59 of it for digits of random sign;
-// an FP64 multiply-add chain rounds its partial sums at 2^-53 each.  The
-// epilogue joins the eight integers into one FP64 number with a single
+// order.  What is cut off and the dropped levels are relative to max_n |a_n|
+// max_n |T~[n][q]|: under n_cheb 2^-56 of it in the worst case, about 2^-59 for
+// digits of random sign.  A multiply-add chain rounds its partial sums, so where
+// T~ rises as a falls the chain keeps more of sum_n |a_n T~[n][q]|: tables rising by
+// 10^3, 10^6 and 10^9 with n, under coefficients falling to nothing, put 8e-16,
+// 7e-13 and 4e-11 of that sum between the two.  The spectra do not see it: every a_n
+// comes from the fit with a rounding of about 2^-53 max |a| of its own, and against
+// quad precision the same calls are off by 5.1e-14, 1.7e-11 and 1.1e-9 by either
+// path.  Tables of Bessel integrals have max |a| max |T~| <= 1.3 sum_n |a_n T~| over the
+// R nodes of a chi (orders 20 to 96, ells to 120; single columns far from R = 1 reach
+// 1.4e3).  The epilogue joins the eight integers into one FP64 number with a single
 // rounding, in integer arithmetic, and the R sum runs in FP64 multiply-adds.
 //
 // Because every level is exact and the R sum has one fixed order, a
