@@ -417,8 +417,8 @@ int blast_test_trip_wait(blast_plan *plan, int tile);
  * The candidates run the caller's representative batch reqs[0..n) (device
  * outputs the call allocates and frees) under the kernel timer; the fastest
  * set stays in the plan for later calls of any batch size.  cache_path
- * (optional) is a text file keyed by GPU name, plan dimensions and cosmology
- * tiles: a key found there is used without timing; a new choice is appended.
+ * (optional) is a text file keyed by GPU name, plan dimensions, R form, cosmology
+ * tiles and how full the last one is: a key found there is used without timing; a new choice is appended.
  * The tuned set never changes a result beyond the summation order of the
  * chi sum.  Errors: BLAST_EINVAL (plan not served by the tensor cores),
  * BLAST_ENOBASIS, BLAST_ENOMEM, and those of blast_cl_batch.

@@ -205,6 +205,13 @@ int launch_fit_nodes(blast_plan *p, const double *Pq, double *c, cudaStream_t s)
 int launch_contract_ns(blast_plan *p, const ReqDev *dreq, const double *c, const int *d_esel, int n_esel, double *Y,
                        cudaStream_t s);
 bool tc_supported(const blast_plan *p);
+// TMEM lane quadrants (of 32) that hold different cosmologies in a batch's last tile of
+// 128: 1, 2 or 4 (3 count as 4).  A tile with fewer than 4 takes less time.
+inline int tc_tail_quadrants(int n)
+{
+    const int last = (n - 1) % 128 + 1;
+    return last <= 32 ? 1 : last <= 64 ? 2 : 4;
+}
 size_t tc_y_bytes(const blast_plan *p, int n, int n_esel);  // R-tile partials of a tensor-core call
 size_t tc_ws_total(const blast_plan *p, int n);  // coefficient slices, scales and chi weights of a call
 int tc_reserve(blast_plan *p, int n);

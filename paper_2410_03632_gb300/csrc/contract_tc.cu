@@ -1028,9 +1028,10 @@ int launch_contract_inst(blast_plan *p, const CUtensorMap &mapB, const CUtensorM
     using C = TcCfg<KC>;
     // persistent CTAs: the autotuned count when set, else every SM.  A last cosmology
     // tile of at most 32 (64) takes less than a full one, measured 1630 (1810) cycles of
-    // 2470 a basis tile at order 64 and 2250 of 2650 at order 96, where the MMAs bound it
-    const int units = args.ngr * args.nqt, nfull = args.nbt - 1, last = args.n - nfull * kM;
-    const double share = last > 64 ? 1.0 : KC == 2 ? 0.85 : last <= 32 ? 0.66 : 0.73;
+    // 2470 a basis tile at order 64 and 2250 of 2650 at order 96, where the MMAs bound it;
+    // other orders take the share of 64 or 96, whichever they share the kernel with
+    const int units = args.ngr * args.nqt, nfull = args.nbt - 1, tail = tc_tail_quadrants(args.n);
+    const double share = tail == 4 ? 1.0 : KC == 2 ? 0.85 : tail == 1 ? 0.66 : 0.73;
     int grid = p->tune.grid > 0 ? p->tune.grid : p->sms;
     if (grid < args.nbt) grid = args.nbt;
     args.cta_full = (int)(grid / (nfull + share));

@@ -4,7 +4,9 @@
 // and stages.  Each candidate runs the caller's representative batch a few
 // times under the plan's kernel timer; the fastest stays in the plan.  A
 // cache file keeps choices across processes, one line per key:
-//   <GPU name>|L|X|n_R|N|max_clust|max_lens|cosmology tiles <TAB> grid W NS
+//   <GPU name>|L|X|n_R|N|max_clust|max_lens|r_form|cosmology tiles|quadrants of the last <TAB> grid W NS
+// The CTAs are dealt to the tiles by cost and the passes may be units of their own, so
+// the count depends on how full the last tile is and on the number of passes.
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -14,7 +16,7 @@
 
 namespace {
 
-std::string tune_key(const blast_plan *p, int nbt)
+std::string tune_key(const blast_plan *p, int nbt, int tail)
 {
     cudaDeviceProp prop;
     std::string name = "gpu";
@@ -22,7 +24,8 @@ std::string tune_key(const blast_plan *p, int nbt)
     for (char &c : name)
         if (c == '|' || c == '\t' || c == '\n') c = '_';
     char buf[256];
-    snprintf(buf, sizeof buf, "|%d|%d|%d|%d|%d|%d|%d", p->L, p->X, p->Rn, p->N, p->max_clust, p->max_lens, nbt);
+    snprintf(buf, sizeof buf, "|%d|%d|%d|%d|%d|%d|%d|%d|%d", p->L, p->X, p->Rn, p->N, p->max_clust, p->max_lens,
+             p->r_form, nbt, tail);
     return name + buf;
 }
 
@@ -73,7 +76,7 @@ extern "C" int blast_autotune(blast_plan *p, int n, const blast_request *reqs, c
     if (!p->havebf) return BLAST_ENOBASIS;
     BL_CUDA(cudaSetDevice(p->device));
     const int nbt = (n + 127) / 128;
-    const std::string key = tune_key(p, nbt);
+    const std::string key = tune_key(p, nbt, tc_tail_quadrants(n));
     int grid = 0, w = 0, ns = 0;
     if (cache_path && cache_lookup(cache_path, key, grid, w, ns)) {
         p->tune.grid = grid; p->tune.red_w = w; p->tune.red_ns = ns; p->tune.nbt = nbt;
@@ -87,12 +90,10 @@ extern "C" int blast_autotune(blast_plan *p, int n, const blast_request *reqs, c
         if (cudaMalloc(&outs[i], bytes) != cudaSuccess) { cudaGetLastError(); rc = BLAST_ENOMEM; }
     }
     cudaStream_t s = (cudaStream_t)stream;
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
-    const int gmax = sms / nbt * nbt;
-    // candidates: every SM and a few counts a cosmology tile below
-    std::vector<int> grids;
-    for (int k = 0; k < 6 && gmax - k * nbt >= nbt; k++) grids.push_back(gmax - k * nbt);
+    // candidates: every SM (the built-in choice; more tiles than SMs: a CTA each) and a few
+    // counts a CTA per cosmology tile below
+    std::vector<int> grids(1, p->sms > nbt ? p->sms : nbt);
+    for (int k = 1; k < 6 && p->sms - k * nbt >= nbt; k++) grids.push_back(p->sms - k * nbt);
     const int Ws[3] = {2, 4, 8};
     double best = 1e300;
     int bg = 0, bw = 0, bns = 0;

@@ -55,3 +55,28 @@ def test_autotune_and_cache(tmp_path):
     finally:
         plan.close()
         plan2.close()
+
+
+def test_cache_tells_batches_of_other_shapes_apart(tmp_path):
+    """The CTAs are dealt by the cost of the tiles, so a last tile of at most 32, of at most 64 and a fuller
+    one are tuned apart, as are the two R forms."""
+    cache = tmp_path / "tune.txt"
+    plans = []
+    try:
+        for sym in (0, 1):
+            spec = synth.plan_spec("tc")
+            spec.r_form = sym
+            plan = bl.Plan(spec)
+            plans.append(plan)
+            plan.precompute(bl.BLAST_BASIS_BF16S)
+            chi, R, _ = plan.nodes()
+            rqs = [synth.config_request("tc", chi, R, i) for i in range(3)]
+            for n in (130, 150, 180, 250):      # two tiles: 2, 22, 52 and 122 cosmologies in the last
+                reqs = [plan.request(rqs[i % 3]) for i in range(n)]
+                assert bl.blast_autotune(plan.h, reqs, cache) == bl.BLAST_OK
+                assert 2 <= bl.blast_tuned_params(plan.h)[0]
+    finally:
+        for plan in plans:
+            plan.close()
+    keys = [line.split("\t")[0] for line in cache.read_text().splitlines()]
+    assert len(keys) == len(set(keys)) == 6     # 130 and 150 share one
