@@ -530,7 +530,7 @@ k_contract_fx(const __grid_constant__ CUtensorMap mapT, const FxArgs A)
                 // even length: the 16 groups, and with them the four FP64 pipes, share the work
                 const int rows = per * most, passes = (rows + 16 * kJC - 1) / (16 * kJC);
                 const int jc = passes ? (rows + 16 * passes - 1) / (16 * passes) : 1;
-                // quotients of small numbers (row < 2^14, divisors <= 32) by multiplication
+                // quotients of small numbers (row < 2^16, divisors <= 32) by multiplication
                 auto decode = [&](int row, int &node, int &b, int &j) {
                     const int nb = inv ? (int)__umulhi(row, inv) : row;
                     j = row - nb * most;

@@ -1,7 +1,7 @@
 """The batch-size and grid rules of the tensor-core and FP32 contractions at
 their edges: cosmology tiles that repeat over the lane quadrants, a partial
 last tile with CTAs of its own, passes as units, fewer tiles than epilogue
-turns, FP32 groups of 1, 4, 8 and 16 cosmologies and every R-node count a thread
+turns, FP32 groups of 4, 8 and 16 cosmologies and every R-node count a thread
 can hold.  A cosmology's bits do not depend on any of it, so each result equals
 the same request evaluated alone, and one of them is held to the FP64 path:
 e_ij <= 1e-4 on the tensor cores (their bar), and for FP32, whose sums of N +
