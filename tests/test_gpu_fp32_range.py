@@ -1,7 +1,7 @@
-"""FP32 batches whose weights lie more than 2^31 floats apart: 16 cosmologies of
-16 + 16 tracers on 11,700 x 128 chi-R nodes (9.3 GB of weights).  A cosmology's
-bits do not depend on its batch, so the first and the last two equal the same
-requests evaluated alone."""
+"""FP32 batches of 16 + 16 tracers whose weights lie more than 2^31 floats apart (9
+to 12 GB of weights), one for every group size and R-node count of the kernel.  A
+cosmology's bits do not depend on its batch, so the first and the last two equal
+the same requests evaluated alone."""
 import types
 
 import numpy as np
@@ -25,10 +25,11 @@ if not _have_gpu():
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
 
-def test_weights_further_apart_than_a_32_bit_offset():
+@pytest.mark.parametrize("X,Rn,n", [(11700, 128, 16), (58600, 128, 4), (12600, 256, 8), (14700, 512, 4), (6300, 512, 8)])
+def test_weights_further_apart_than_a_32_bit_offset(X, Rn, n):
     import torch
 
-    X, Rn, n, ng, ns = 11700, 128, 16, 16, 16
+    ng, ns = 16, 16
     Q = X * Rn
     per = 3 * (ng + ns) * (X + Q)          # floats of work space a request
     assert (n - 1) * per > 2 ** 31
