@@ -617,7 +617,8 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
 // every entry that can matter: all entries finite, and no (type, ell) whose
 // largest entry is under 2^-700 (columns under 2^-953 are taken as zero; a
 // whole table that small keeps the CUDA-core kernel, as does a table with
-// infinities or NaN, whose sums follow the rules of FP64 there).
+// infinities or NaN, whose sums follow the rules of FP64 there), and the memory
+// for the exponents (2 bytes a column beside 8 n_cheb of the table) is to be had.
 int fx_prepare(blast_plan *p, cudaStream_t s)
 {
     p->fx_ok = false;
@@ -625,12 +626,12 @@ int fx_prepare(blast_plan *p, cudaStream_t s)
     if (!p->colexp && cudaMalloc(&p->colexp, nslab * p->Q * sizeof(uint16_t)) != cudaSuccess) {
         cudaGetLastError();
         p->colexp = nullptr;
-        return BLAST_ENOMEM;
+        return BLAST_OK;
     }
     if (!p->d_slab && cudaMalloc(&p->d_slab, nslab * sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         p->d_slab = nullptr;
-        return BLAST_ENOMEM;
+        return BLAST_OK;
     }
     BL_CUDA(cudaMemsetAsync(p->d_slab, 0, nslab * sizeof(int), s));
     k_column_exp<<<dim3((p->Q + 255) / 256, (unsigned)nslab), 256, 0, s>>>(p->T64, p->N, p->Q, p->colexp, p->d_slab);
